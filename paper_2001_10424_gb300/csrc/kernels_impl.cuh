@@ -94,6 +94,23 @@ __device__ __forceinline__ T const_row(const Lvl& L, T b, T xf, T acc, bool gd, 
   return fma(wkd, xf, t);
 }
 
+// M row of a constant-viscosity face beside a wall of a tangential axis: w is
+// its link-by-link W row. Explicit roundings, so that every kernel that forms
+// this row (tile, shell, V-cycle legs) gets the same bits.
+template <typename T>
+__device__ __forceinline__ T wall_row(T w, T ws, bool gd, T g2, T dp, T dm) {
+  const T m = mul_rn(w, ws);
+  return gd ? fma(g2, dp - dm, m) : m;
+}
+
+// the Chebyshev direction ca z + cb d (first: ca z) where the stencil is not
+// already scaled by ca, with explicit roundings for the same reason
+template <typename T>
+__device__ __forceinline__ T cheb_wall(T ca, T z, T cb, T dold, bool first) {
+  const T t = mul_rn(ca, z);
+  return first ? t : fma(cb, dold, t);
+}
+
 // W row for variable viscosity at a deep-interior face (all links regular,
 // all cells in the domain): the same operations in the same order as the
 // general link-by-link row, without its bookkeeping. xc points at the face,
@@ -312,8 +329,7 @@ __device__ __forceinline__ void mac_tile_body(const Blk& B, const Lvl& L, int wo
           fused = true;                                                          \
           m = const_row<T, MODE>(L, (MODE == 0) ? b[id] : (T)0, xf, nb_sum<T>(L, x + id), gd, DPLUS, DMINUS); \
         } else {                                                                 \
-          m = w_row<T, false, C>(L, x, p, xf) * Kc<T>::ws(L);                    \
-          if (gd) m += g2 * ((DPLUS) - (DMINUS));                                \
+          m = wall_row<T>(w_row<T, false, C>(L, x, p, xf), Kc<T>::ws(L), gd, g2, gd ? (DPLUS) : (T)0, gd ? (DMINUS) : (T)0); \
         }                                                                        \
       }                                                                          \
       val = (MODE == 0 && !fused) ? b[id] - m : m;                               \
@@ -560,8 +576,7 @@ __device__ __forceinline__ double mac3_shell_body(const Lvl& L, int wonly, const
       if (const_regular<C>(L, p)) {                                                            \
         val = const_row<T, MODE>(L, bb, xf, nb_sum<T>(L, x + id), gd, d0, dm);                 \
       } else {                                                                                 \
-        T m = w_row<T, false, C>(L, x, p, xf) * Kc<T>::ws(L);                                  \
-        if (gd) m += g2 * (d0 - dm);                                                           \
+        const T m = wall_row<T>(w_row<T, false, C>(L, x, p, xf), Kc<T>::ws(L), gd, g2, d0, dm); \
         val = (MODE == 0) ? bb - m : m;                                                        \
       }                                                                                        \
       if (DOT) dot += (double)xf * (double)val;                                                \
@@ -1190,7 +1205,7 @@ __device__ __forceinline__ T fold2_apply(const Lvl& L, const T* GKB_RESTRICT r, 
   const int P = L.P;
   const T* ra = r + L.off[0] + cb;
   const T* rb = r + L.off[1] + cb;
-  T acc = f(0) * GKB_LDG(C == 0 ? ra : rb);
+  T acc = mul_rn(f(0), GKB_LDG(C == 0 ? ra : rb));
   const T* base[6];
   int o[6];
   if (C == 0) {
@@ -1203,15 +1218,24 @@ __device__ __forceinline__ T fold2_apply(const Lvl& L, const T* GKB_RESTRICT r, 
 #pragma unroll
   for (int u = 0; u < 6; ++u) {
     const T c = f(1 + u);
-    if (Inner || c != (T)0) acc += c * GKB_LDG(base[u] + o[u]);
+    if (Inner || c != (T)0) acc = fma(c, GKB_LDG(base[u] + o[u]), acc);
   }
   return acc;
 }
 
+// the positions whose step uses the interior stencils already scaled by ca
+// (d = z + cb d): those of the 32 x 8 blocks of k_cheb2 that lie wholly in the
+// interior class. A rule per block, not per position: on the FP64 pipe a warp
+// that ran both forms would pay for both (7 % of a 1024^2 solve).
+__device__ __forceinline__ bool cheb2_scaled(const Lvl& L, int i, int j) {
+  const int i0 = i & ~(BX - 1), j0 = j & ~(BY - 1);
+  return i0 >= 3 && i0 + BX - 1 <= L.n[0] - 3 && j0 >= 3 && j0 + BY - 1 <= L.n[1] - 3;
+}
+
 // one Chebyshev step of the 2D constant-viscosity smoother through the class
-// stencils (levels with at least six cells per axis). Blocks whose positions
-// are all interior use the kernel parameter's stencils, already scaled by
-// ca (d = z + cb d); the others each position's class stencil from the table.
+// stencils (levels with at least six cells per axis): the kernel parameter's
+// scaled stencils where cheb2_scaled, else each position's class stencil from
+// the table.
 template <typename T>
 __device__ __forceinline__ void cheb2_body(const Blk& B, const Lvl& L, const T* GKB_RESTRICT r, T* GKB_RESTRICT x,
                                            T* GKB_RESTRICT d, T ca, T cb, int x_zero, const T* GKB_RESTRICT table,
@@ -1219,8 +1243,8 @@ __device__ __forceinline__ void cheb2_body(const Blk& B, const Lvl& L, const T* 
   const int i0 = B.x * BX, j0 = B.y * BY;
   const int i = i0 + threadIdx.x, j = j0 + threadIdx.y;
   const int P = L.P;
-  if (i0 >= 3 && i0 + BX - 1 <= L.n[0] - 3 && j0 >= 3 && j0 + BY - 1 <= L.n[1] - 3) {
-    const int p0 = j * P + i;
+  const int p0 = j * P + i;
+  if (cheb2_scaled(L, i0, j0)) {
 #define GKB_CHEB2_IN(C)                                                                  \
     {                                                                                    \
       const int id = (int)L.off[C] + p0;                                                 \
@@ -1238,7 +1262,6 @@ __device__ __forceinline__ void cheb2_body(const Blk& B, const Lvl& L, const T* 
   }
   if (i > L.n[0] || j > L.n[1]) return;
   const int pc = cls7(i, L.n[0]) * 7 + cls7(j, L.n[1]);
-  const int p0 = j * P + i;
   const T* fold = table + FOLD3_OFF + (size_t)pc * 48;
 #define GKB_CHEB2(C)                                                                              \
   if (in_store<C>(L, i, j, 0) && face_active<C>(L, i, j, 0)) {                                    \
@@ -1246,7 +1269,7 @@ __device__ __forceinline__ void cheb2_body(const Blk& B, const Lvl& L, const T* 
     const T dold = (cb != (T)0) ? d[id] : (T)0;                                                   \
     const T xold = x_zero ? (T)0 : x[id];                                                         \
     const T z = fold2_apply<T, C, false>(L, r, p0, [&](int q) { return GKB_LDG(fold + C * 16 + q); }); \
-    const T dn = (cb != (T)0) ? ca * z + cb * dold : ca * z;                                      \
+    const T dn = cheb_wall<T>(ca, z, cb, dold, cb == (T)0);                                       \
     d[id] = dn;                                                                                   \
     x[id] = x_zero ? dn : xold + dn;                                                              \
   }

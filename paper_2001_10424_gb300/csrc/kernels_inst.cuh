@@ -197,6 +197,12 @@ void Ops<KT>::restrict_(const Lvl& Lf, const Lvl& Lc, const KT* rf, KT* bc, KT* 
 }
 
 template <>
+void Ops<KT>::restrict_slopes(const Lvl& Lc, const KT* tmp, KT* bc, cudaStream_t s) {
+  ProfScope ps_(GKB_KC_RESTRICT, s, lvl_unknowns(Lc));
+  k_restrict_flux2d_b<KT><<<face_grid(Lc), dim3(BX, BY), 0, s>>>(Lc, tmp, bc);
+}
+
+template <>
 void Ops<KT>::coarse(int m, const KT* Minv, const int* idx, const KT* b, KT* x, cudaStream_t s) {
   ProfScope ps_(GKB_KC_COARSE, s, (long long)m);
   const int warps_per_block = 8;

@@ -38,6 +38,7 @@
 #include "../../include/gkb.h"
 #include "gkb_device.cuh"
 #include "kernels_impl.cuh"
+#include "legs.cuh"
 #include "lockstep.cuh"
 #include "solver.cuh"
 
@@ -129,6 +130,15 @@ struct JProl { JobHead h; Lvl Lf, Lc; const T* xc; T* xf; };
 template <typename T>
 __global__ void __launch_bounds__(BX* BY) kb_prolong(const JProl<T>* jobs, const unsigned* map) {
   LS_RUN(JProl<T>, prolong_flux2d_body<T>(B, job.Lf, job.Lc, job.xc, job.xf))
+}
+
+// a level's fused down or up leg (legs.cuh)
+template <typename T>
+struct JLeg { JobHead h; LegArgs<T> A; };
+template <typename T, int DEG, int KIND, bool DOWN>
+__global__ void __launch_bounds__(LegShape<DEG, KIND, DOWN>::NT) kb_leg(const JLeg<T>* jobs, const unsigned* map) {
+  extern __shared__ __align__(16) unsigned char leg_sm[];
+  LS_RUN(JLeg<T>, leg_body<T, DEG, KIND, DOWN>(B, job.A, (T*)leg_sm))
 }
 
 template <typename T>
@@ -433,7 +443,7 @@ struct Lockstep::Impl {
   // p's job (head flags included) and returns its own launch grid
   template <class J, class Make>
   void launch(cudaStream_t st, int kc, const std::vector<int>& ps, dim3 block, Make make,
-              void (*kern)(const J*, const unsigned*)) {
+              void (*kern)(const J*, const unsigned*), size_t smem = 0) {
     std::vector<J> jobs;
     std::vector<unsigned> map;
     unsigned first = 0;
@@ -454,7 +464,7 @@ struct Lockstep::Impl {
     if (jobs.empty()) return;
     const J* dj = put(jobs);
     const unsigned* dm = put_map(map);
-    kern<<<first, block, 0, st>>>(dj, dm);
+    kern<<<first, block, smem, st>>>(dj, dm);
     GKB_CUDA(cudaGetLastError());
     cl[sect][kc] += 1;
   }
@@ -532,6 +542,44 @@ struct Lockstep::Impl {
     }
   }
 
+  // one leg of the problems `ps` at depth d, which all take the same tiling
+  template <typename T, int DEG, int KIND, bool DOWN>
+  void leg_launch(cudaStream_t st, const std::vector<int>& ps, int d, const int* F,
+                  const std::function<const T*(int)>& r0, const std::function<T*(int)>& z0) {
+    using G = LegShape<DEG, KIND, DOWN>;
+    constexpr size_t sm = G::template smem<T>();
+    if (sm > 48 * 1024)
+      GKB_CUDA(cudaFuncSetAttribute(kb_leg<T, DEG, KIND, DOWN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    launch<JLeg<T>>(st, GKB_KC_SMOOTH, ps, dim3(G::NT), [&](int p, JLeg<T>& j) {
+      const Gmg<T>& M = gmg<T>(p);
+      const bool split = d > 0 && M.leg_on(d - 1);  // as in Gmg<T>::vcycle
+      j.h.active = F + p;
+      const T* b = d == 0 ? r0(p) : (!DOWN && split) ? M.lev[d].d.p : M.lev[d].b.p;
+      gmg_leg_args<T>(M, d, b, DOWN && split ? M.lev[d].x.p : nullptr, d == 0 ? z0(p) : nullptr, j.A);
+      return G::grid(j.A.L);
+    }, kb_leg<T, DEG, KIND, DOWN>, sm);
+  }
+  template <typename T, int DEG, bool DOWN>
+  void leg_kinds(cudaStream_t st, const std::vector<int>& ps, int d, const int* F,
+                 const std::function<const T*(int)>& r0, const std::function<T*(int)>& z0) {
+    auto of = [&](int kind) {
+      std::vector<int> v;
+      for (int p : ps)
+        if (gmg<T>(p).lev[d].leg == kind) v.push_back(p);
+      return v;
+    };
+    leg_launch<T, DEG, LEG_8, DOWN>(st, of(LEG_8), d, F, r0, z0);
+    if constexpr (sizeof(T) == 4) leg_launch<T, DEG, LEG_STRIP, DOWN>(st, of(LEG_STRIP), d, F, r0, z0);
+  }
+  template <typename T, bool DOWN>
+  void legs(cudaStream_t st, const std::vector<int>& ps, int d, const int* F,
+            const std::function<const T*(int)>& r0, const std::function<T*(int)>& z0) {
+    const int deg = ps.empty() ? 0 : gmg<T>(ps[0]).degree;
+    if (deg == 1) leg_kinds<T, 1, DOWN>(st, ps, d, F, r0, z0);
+    else if (deg == 2) leg_kinds<T, 2, DOWN>(st, ps, d, F, r0, z0);
+    else if (deg == 3) leg_kinds<T, 3, DOWN>(st, ps, d, F, r0, z0);
+  }
+
   // z = B r on the finest level of every problem (r0(p), z0(p) its arrays)
   template <typename T>
   void vcycle(cudaStream_t st, const int* F, const std::function<const T*(int)>& r0,
@@ -548,9 +596,30 @@ struct Lockstep::Impl {
         if ((int)gmg<T>(p).lev.size() - 1 > d) v.push_back(p);
       return v;
     };
+    auto pick = [&](const std::vector<int>& v, int d, bool fused) {
+      std::vector<int> w;
+      for (int p : v)
+        if (gmg<T>(p).leg_on(d) == fused) w.push_back(p);
+      return w;
+    };
     for (int d = 0; d < dmax; ++d) {
-      const std::vector<int> ps = deeper(d);
-      if (ps.empty()) break;
+      const std::vector<int> level = deeper(d);
+      if (level.empty()) break;
+      // levels with fused legs; where the next level has none, the transposed
+      // slopes' own pass completes its right-hand side
+      const std::vector<int> fs = pick(level, d, true);
+      legs<T, true>(st, fs, d, F, r0, z0);
+      launch<JRestr<T>>(st, GKB_KC_RESTRICT, pick(fs, d + 1, false), dim3(BX, BY), [&](int p, JRestr<T>& j) {
+        auto& G = gmg<T>(p);
+        j.h.active = F + p;
+        j.Lf = G.lev[d].L;
+        j.Lc = G.lev[d + 1].L;
+        j.bc = G.lev[d + 1].b.p;
+        j.tmp = G.lev[d + 1].x.p;
+        return face_grid(j.Lc);
+      }, kb_restr_b<T>);
+      const std::vector<int> ps = pick(level, d, false);
+      if (ps.empty()) continue;
       const auto bf = lb(d);
       const auto xf = lx(d);
       smooth<T>(st, ps, d, F, bf, xf, true);
@@ -596,7 +665,9 @@ struct Lockstep::Impl {
       return dim3((G.coarse_m + 7) / 8);
     }, kb_coarse<T>);
     for (int d = dmax - 1; d >= 0; --d) {
-      const std::vector<int> ps = deeper(d);
+      const std::vector<int> level = deeper(d);
+      legs<T, false>(st, pick(level, d, true), d, F, r0, z0);
+      const std::vector<int> ps = pick(level, d, false);
       if (ps.empty()) continue;
       const auto bf = lb(d);
       const auto xf = lx(d);

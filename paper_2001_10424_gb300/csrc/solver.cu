@@ -554,6 +554,7 @@ void Gmg<T>::build(const Lvl& fine, const T* fine_mu, int coarse_max, int deg, c
   GKB_CUDA(cudaMemcpyAsync(coarse_idx.p, idx32.data(), m * sizeof(int), cudaMemcpyHostToDevice, s));
   GKB_CUDA(cudaStreamSynchronize(s));
   gmg_tail_setup<T>(*this, tail_side, s);
+  gmg_leg_plan<T>(*this);
 }
 
 template <typename T>
@@ -616,7 +617,20 @@ void Gmg<T>::vcycle(const T* r0, T* z0, cudaStream_t s, bool use_net) {
   // the fused coarse end: levels from tail_level on run in one cluster kernel
   const bool tail = !with_net && tail_level > 0 && tail_buf.p;
   const int ld = tail ? tail_level : lc;  // levels handled by separate launches
+  // levels whose steps run as two fused kernels; the composite network's
+  // level starts from the network's correction, which the legs do not
+  auto fused = [&](int l) { return l < ld && leg_on(l) && !(with_net && l == net_level); };
+  // a fused level leaves its coarse right-hand side as (rU, rD) in (b, x);
+  // the next fused level completes it as it loads it (into d), any other
+  // level by the transposed slopes' own pass
+  auto leg_b = [&](int l) { return (l > 0 && fused(l - 1)) ? (const T*)lev[l].d.p : lvl_b(l); };
   for (int l = 0; l < ld; ++l) {
+    if (fused(l)) {
+      const bool split = l > 0 && fused(l - 1);
+      gmg_leg<T>(*this, l, true, lvl_b(l), split ? (const T*)lev[l].x.p : nullptr, z0, s);
+      if (!fused(l + 1)) Ops<T>::restrict_slopes(lev[l + 1].L, lev[l + 1].x.p, lev[l + 1].b.p, s);
+      continue;
+    }
     bool x_zero = true;
     if (with_net && l == net_level) {  // composite form
       net_at(l);
@@ -630,6 +644,10 @@ void Gmg<T>::vcycle(const T* r0, T* z0, cudaStream_t s, bool use_net) {
   else if (replace) net_at(lc);
   else Ops<T>::coarse(coarse_m, coarse_inv.p, coarse_idx.p, lvl_b(lc), lvl_x(lc), s);
   for (int l = ld - 1; l >= 0; --l) {
+    if (fused(l)) {
+      gmg_leg<T>(*this, l, false, leg_b(l), nullptr, z0, s);
+      continue;
+    }
     Ops<T>::prolong(lev[l].L, lev[l + 1].L, lev[l + 1].x.p, lvl_x(l), lev[l + 1].sl.p, s);
     smooth(l, lvl_b(l), lvl_x(l), false, s);
   }
@@ -1133,8 +1151,7 @@ void Solver::set_problem(const gkb_grid* g, const double* viscosity, double mu0_
   }
   L64.mu0 = viscosity ? 1.0 : mu0;
   L64.sym = symgrad ? 1 : 0;
-  // fast paths: measured faster in FP32, slower in FP64 (FP64-pipe bound)
-  L64.fast = (opt.kernel_variant == 2) ? 1 : 0;
+  L64.fast = fast64() ? 1 : 0;
   finish_level(L64);
   Compact cmp = make_compact(L64);
   m = cmp.m;
@@ -1254,18 +1271,27 @@ void Solver::set_problem(const gkb_grid* g, const double* viscosity, double mu0_
   stats.setup_seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
 }
 
+// Deep-interior fast paths on FP64 levels: kernel_variant 1 nowhere, 2
+// everywhere, 0 where they measured faster: the 2D constant-viscosity class
+// stencils and fused legs (1024^2 solve 319 -> 265 ms, 64^2 50 -> 27 ms), not
+// variable viscosity (1024^2 418 ms without, 508 ms with) and not 3D (64^3
+// 638 ms without, 863 ms with)
+bool Solver::fast64() const {
+  if (opt.kernel_variant != 0) return opt.kernel_variant == 2;
+  return grid.dim == 2 && !mu64.p;
+}
+
 // Multigrid hierarchy and CG of the handle's precision from the current
 // options (smoother degree, coarse size, kernel variant).
 void Solver::build_inner() {
   const bool mixed = opt.precision == GKB_PREC_MIXED;
   const bool use_gmg = opt.inner == GKB_INNER_GMG_PCG || opt.inner == GKB_INNER_FGMRES || learned_inner();
-  // deep-interior fast paths: variant 0 enables them in FP32 only (faster
-  // there, slower on the FP64 pipe), 1 nowhere, 2 everywhere
-  L64.fast = (opt.kernel_variant == 2) ? 1 : 0;
+  L64.fast = fast64() ? 1 : 0;
   L32.fast = (opt.kernel_variant == 1) ? 0 : 1;
   gmg32.cheb_lo = gmg64.cheb_lo = opt.cheb_lo;
   gmg32.cheb_hi = gmg64.cheb_hi = opt.cheb_hi;
   gmg32.tail_side = gmg64.tail_side = opt.tail_side;
+  gmg32.legs = gmg64.legs = !opt.profile;
   if (mixed) {
     if (use_gmg) gmg32.build(L32, mu32.p, opt.coarse_max, opt.smoother_degree, red, scal.p, stream);
     cg32.init(L32, use_gmg ? &gmg32 : nullptr, red, cg_dev, cg_host);

@@ -83,6 +83,7 @@ struct Gmg {
     std::vector<double> ca, cb; // Chebyshev coefficients per step
     std::vector<double> fold_in; // constant viscosity: the interior class stencils (host copy)
     double lam_max = 0;
+    int leg = 0;                // tiling of the fused legs (LegKind, legs.cuh), 0: separate launches
   };
   std::vector<Level> lev;
   DevBuf<T> coarse_inv;
@@ -105,9 +106,12 @@ struct Gmg {
   // viscosity): levels from tail_level on (the first whose longer side is at
   // most tail_side) run inside k_vtail; -1: off
   int tail_side = 0;
+  bool legs = true;   // fused legs where a level qualifies (off while profiling: every step its own launch)
   int tail_level = -1;
   int tail_cs = 0;
   DevBuf<unsigned char> tail_buf;
+  // level l's steps run as fused legs (false past the last level)
+  bool leg_on(int l) const { return legs && l < (int)lev.size() && lev[l].leg > 0; }
   void attach_net(Unet* u, int level, bool composite, cudaStream_t s);
   void detach_net();
   Gmg() = default;
@@ -128,6 +132,17 @@ template <typename T>
 void gmg_tail_setup(Gmg<T>& G, int side, cudaStream_t s);
 template <typename T>
 void gmg_tail_launch(const Gmg<T>& G, cudaStream_t s);
+
+// the fused V-cycle legs (legs.cu): which levels take them; the launch of
+// level l's down or up leg (b: its right-hand side, or with rd the gathered
+// part of it; z0: the finest level's result)
+template <typename T> struct LegArgs;
+template <typename T>
+void gmg_leg_plan(Gmg<T>& G);
+template <typename T>
+void gmg_leg_args(const Gmg<T>& G, int l, const T* b, const T* rd, T* z0, LegArgs<T>& A);
+template <typename T>
+void gmg_leg(const Gmg<T>& G, int l, bool down, const T* b, const T* rd, T* z0, cudaStream_t s);
 
 // An instantiated graph of a whole solve with the launch counts of its
 // parts recorded at capture time: [0] once, [1] per outer iteration,
@@ -248,6 +263,7 @@ struct Solver {
   bool learned_inner() const { return opt.inner == GKB_INNER_FCG_UNET || opt.inner == GKB_INNER_FCG_UNET_MG; }
   void set_net(Unet* u);
   double tuned_ms = 0;            // inner-solve time of the tuned configuration
+  bool fast64() const;
   void build_inner();
   double time_inner_solve(int* its = nullptr);  // device ms of one inner solve (best of 3)
   void autotune_inner(bool var_mu, int weighted);
