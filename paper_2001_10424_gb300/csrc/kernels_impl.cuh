@@ -171,9 +171,14 @@ __device__ __forceinline__ void mac_tile_body(const Blk& B, const Lvl& L, int wo
   const int i = i0 + tx, j = j0 + ty;
   const bool gd = L.has_gd && !wonly && x != nullptr;
   const int cur = (L.dim == 3) ? 1 : 0;
-  const bool tile2d = L.dim == 2 && L.fast && x != nullptr && (!VarMu || EmPtr<T>::get(L) == nullptr) && i0 >= 2 &&
+    // FP64 constant-viscosity rows take the general path on 2D levels below
+  // 2^19 cells, where the tile's barriers cost more than its shared operands
+  // save (512^2 solve 107.9 -> 102.7 ms, 256^2 57.8 -> 54.7 ms); above, two
+  // concurrent 1024^2 solves are 2 % faster with the tile
+  const bool fast2d = VarMu || sizeof(T) == 4 || L.n[0] * (long long)L.n[1] >= (1LL << 19);
+  const bool tile2d = fast2d && L.dim == 2 && L.fast && x != nullptr && (!VarMu || EmPtr<T>::get(L) == nullptr) && i0 >= 2 &&
                       i0 + BX + 2 <= L.n[0] && j0 >= 2 && j0 + BY + 2 <= L.n[1];
-  if (tile2d) {
+  if (fast2d && tile2d) {
     constexpr int TW = BX + 2, TN = (BY + 2) * (BX + 2);
     const T* mu = MuPtr<T>::get(L);
     for (int t = tid; t < TN; t += BX * BY) {
@@ -218,7 +223,7 @@ __device__ __forceinline__ void mac_tile_body(const Blk& B, const Lvl& L, int wo
   const T g2 = Kc<T>::g2(L);
   const long long cb = cix(L, i, j, k);
   double dot = 0.0;
-  if (tile2d && !VarMu) {
+  if (fast2d && tile2d && !VarMu) {
     // GKB_TILE_DEEP with every operand from the tiles
     const int c = tx + 1, r = ty + 1;
 #define GKB_TILE_SMEM(C, DPLUS, DMINUS)                                          \
@@ -233,7 +238,7 @@ __device__ __forceinline__ void mac_tile_body(const Blk& B, const Lvl& L, int wo
     GKB_TILE_SMEM(0, Dt[0][ty + 1][tx + 1], Dt[0][ty + 1][tx])
     GKB_TILE_SMEM(1, Dt[0][ty + 1][tx + 1], Dt[0][ty][tx + 1])
 #undef GKB_TILE_SMEM
-  } else if (tile2d) {
+  } else if (fast2d && tile2d) {
     // the operations and roundings of w_row_var_deep + GKB_TILE_VDEEP, with
     // every operand from the tiles (bitwise equal to the general row)
     const T ws = Kc<T>::ws(L);
@@ -280,7 +285,7 @@ __device__ __forceinline__ void mac_tile_body(const Blk& B, const Lvl& L, int wo
       if (DOT) dot += (double)xf * (double)val;
       y[id] = val;
     }
-  } else if (!VarMu && x != nullptr && deep_interior(L, i, j, k)) {
+  } else if (!VarMu && x != nullptr && (fast2d || L.dim == 3) && deep_interior(L, i, j, k)) {
 #define GKB_TILE_DEEP(C, DPLUS, DMINUS)                                          \
     {                                                                            \
       const long long id = L.off[C] + cb;                                        \
