@@ -794,6 +794,13 @@ __host__ __device__ __forceinline__ int sym4(int r, int c) {
   return r <= c ? (r * (7 - r)) / 2 + c : (c * (7 - c)) / 2 + r;
 }
 
+// one row of a patch inverse times the patch residual, with explicit roundings
+// (the fused legs form the same sums)
+template <typename T>
+__device__ __forceinline__ T patch_dot(T t0, T t1, T t2, T t3, T r0, T r1, T r2, T r3) {
+  return fma(t3, r3, fma(t2, r2, fma(t1, r1, mul_rn(t0, r0))));
+}
+
 // row `slot` of the stored inverse of patch e applied to the patch residual
 template <typename T, int E>
 __device__ __forceinline__ T patch_vtab_row(const Lvl& L, const T* r, const int e[3], long long ce, int slot,
@@ -806,8 +813,8 @@ __device__ __forceinline__ T patch_vtab_row(const Lvl& L, const T* r, const int 
   // faces outside the store (below the first node) are inactive: coefficient 0
   const T r0 = e[b] > 0 ? GKB_LDG(ra - strd<b>(L)) : (T)0;
   const T r2 = e[a] > 0 ? GKB_LDG(rb - strd<a>(L)) : (T)0;
-  return GKB_LDG(t + sym4(slot, 0) * Q) * r0 + GKB_LDG(t + sym4(slot, 1) * Q) * GKB_LDG(ra) +
-         GKB_LDG(t + sym4(slot, 2) * Q) * r2 + GKB_LDG(t + sym4(slot, 3) * Q) * GKB_LDG(rb);
+  return patch_dot<T>(GKB_LDG(t + sym4(slot, 0) * Q), GKB_LDG(t + sym4(slot, 1) * Q), GKB_LDG(t + sym4(slot, 2) * Q),
+                      GKB_LDG(t + sym4(slot, 3) * Q), r0, GKB_LDG(ra), r2, GKB_LDG(rb));
 }
 
 // contribution of the patch of edge e (padded index ce) to slot `slot` of z = C r
@@ -1537,7 +1544,7 @@ __device__ __forceinline__ void cheb_body(const Blk& B, const Lvl& L, const T* G
   if (in_store<C>(L, i, j, k) && face_active<C>(L, i, j, k)) {                   \
     const long long id = L.off[C] + pc;                                          \
     const T z = patch_apply<T, VarMu, C>(L, r, p, pc, table);                    \
-    const T dn = (cb != (T)0) ? ca * z + cb * d[id] : ca * z;                    \
+    const T dn = cheb_wall<T>(ca, z, cb, (cb != (T)0) ? d[id] : (T)0, cb == (T)0); \
     d[id] = dn;                                                                  \
     x[id] = x_zero ? dn : x[id] + dn;                                            \
   }

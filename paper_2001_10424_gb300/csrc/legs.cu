@@ -5,7 +5,7 @@
 namespace gkb {
 
 template <typename T, int DEG, int KIND, bool DOWN>
-__global__ void __launch_bounds__(LegShape<DEG, KIND, DOWN>::NT, KIND == LEG_STRIP ? 2 : 1)
+__global__ void __launch_bounds__(LegShape<DEG, KIND, DOWN>::NT, KIND == LEG_8 ? 1 : 2)
     k_leg(const __grid_constant__ LegArgs<T> A) {
   extern __shared__ __align__(16) unsigned char leg_sm[];
   leg_body<T, DEG, KIND, DOWN>(native_blk(), A, (T*)leg_sm);
@@ -27,6 +27,7 @@ template <typename T, int DEG, bool DOWN>
 void launch_kind(int kind, const LegArgs<T>& A, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
     if (kind == LEG_STRIP) return launch_leg<T, DEG, LEG_STRIP, DOWN>(A, s);
+    if (kind == LEG_VAR) return launch_leg<T, DEG, LEG_VAR, DOWN>(A, s);
   }
   launch_leg<T, DEG, LEG_8, DOWN>(A, s);
 }
@@ -72,7 +73,7 @@ void gmg_leg_args(const Gmg<T>& G, int l, const T* b, const T* rd, T* z0, LegArg
   for (int k = 0; k < G.degree; ++k) {
     A.ca[k] = (T)V.ca[k];
     A.cb[k] = (T)V.cb[k];
-    A.fs[k] = fold2_scaled<T>(V.fold_in.data(), (double)(T)V.ca[k]);
+    if (!V.fold_in.empty()) A.fs[k] = fold2_scaled<T>(V.fold_in.data(), (double)(T)V.ca[k]);
   }
 }
 template void gmg_leg_args<float>(const Gmg<float>&, int, const float*, const float*, float*, LegArgs<float>&);
@@ -83,8 +84,10 @@ void gmg_leg_plan(Gmg<T>& G) {
   for (size_t l = 0; l < G.lev.size(); ++l) {
     auto& V = G.lev[l];
     V.leg = LEG_OFF;
-    if (l + 1 < G.lev.size() && !V.fold_in.empty() && cheb2_level(V.L) && G.degree <= LEG_MAX_DEG)
-      V.leg = leg_kind<T>(V.L);
+    if (l + 1 == G.lev.size() || V.L.dim != 2 || !V.L.fast || G.degree > LEG_MAX_DEG) continue;
+    if (!V.fold_in.empty() && cheb2_level(V.L)) V.leg = leg_kind<T>(V.L);
+    // FP32 variable viscosity with N = n I and the Laplacian form
+    else if (sizeof(T) == 4 && V.L.mu32 && !V.L.nw32 && !V.L.sym) V.leg = LEG_VAR;
   }
 }
 template void gmg_leg_plan<float>(Gmg<float>&);

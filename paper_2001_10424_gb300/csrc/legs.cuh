@@ -434,8 +434,10 @@ struct StripTile {
   static constexpr int TW = EW - HL - HH, TH = EH - HL - HH;  // owned cells
   static constexpr int PAD = EW + 32;                          // neighbours of the tile's rim read here
   static constexpr int PS = EN + PAD;
+  // iterate and residual planes, then the class stencils (constant viscosity)
+  // or the cell viscosities
   template <typename T>
-  static constexpr size_t smem() { return (size_t)(4 * PS + PAD + LEG_FOLD) * sizeof(T); }
+  static constexpr size_t smem(bool var) { return (size_t)(4 * PS + PAD + (var ? PS : LEG_FOLD)) * sizeof(T); }
   static_assert(TW % 2 == 0 && TH % 2 == 0 && TW > 0 && TH > 0, "tiles own whole coarse cells");
 };
 
@@ -608,8 +610,152 @@ struct Strip {
       if (act_v(k)) y[ov + id] = b[k];
     }
   }
-  __device__ __forceinline__ void load_fold(const LegArgs<T>& A) const {
+  __device__ __forceinline__ void setup(const LegArgs<T>& A) const {
     for (int t = IN ? LEG_FOLD : (int)threadIdx.x; t < LEG_FOLD; t += G::NT) fold[t] = leg_fold_entry(A, t);
+  }
+};
+
+// Variable viscosity: the plane after the residual holds the cells' viscosity
+// (0 outside the domain), from which every link forms its node mean; the
+// smoother reads the patch inverses (10 planes of A.table) once per step, and
+// the tile's 40 bytes per node stay in L1 between the steps. The operations
+// are those of the general variable-viscosity row (w_row) and of k_cheb.
+template <typename T, class G, bool IN>
+struct StripVar : Strip<T, G, IN> {
+  using S = Strip<T, G, IN>;
+  using S::X0; using S::X1; using S::R0; using S::R1; using S::i; using S::j; using S::o; using S::nx; using S::ny;
+  using S::xu; using S::xv; using S::bu; using S::bv; using S::du; using S::dv; using S::ru; using S::rv;
+  static constexpr int EW = G::EW, K = G::K;
+  T* MU;
+  __device__ __forceinline__ StripVar(const Lvl& L, int i0, int j0, T* sm) : S(L, i0, j0, sm) { MU = S::fold; }
+  __device__ __forceinline__ void setup(const LegArgs<T>& A) const {
+    const T* mu = MuPtr<T>::get(A.L);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const bool ok = IN || (i >= 0 && i < nx && j + k >= 0 && j + k < ny);
+      MU[o + k * EW] = ok ? GKB_LDG(mu + (j + k) * A.L.P + i) : (T)0;
+    }
+  }
+
+  __device__ __forceinline__ void residual(const Lvl& L) {
+    const bool gd = L.has_gd;
+    const T g2 = Kc<T>::g2(L), ws = Kc<T>::ws(L);
+    T cu[K + 2], cv[K + 2], rr[K + 1], lv[K + 1];  // as in Strip
+    T cm[K + 2], lm[K + 2];                        // viscosity of rows -1 .. K, own column and the one left of it
+    cu[0] = X0[o - EW];
+    cv[0] = X1[o - EW];
+    cu[K + 1] = X0[o + K * EW];
+    cv[K + 1] = X1[o + K * EW];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      cu[k + 1] = xu[k];
+      cv[k + 1] = xv[k];
+    }
+#pragma unroll
+    for (int k = 0; k <= K; ++k) {
+      rr[k] = X0[o + (k - 1) * EW + 1];
+      lv[k] = X1[o + k * EW - 1];
+    }
+#pragma unroll
+    for (int k = 0; k < K + 2; ++k) {
+      cm[k] = MU[o + (k - 1) * EW];
+      lm[k] = MU[o + (k - 1) * EW - 1];
+    }
+    // node means as edge_mu_cells sums them, per component: over the cells at
+    // (C-1, A-1), (C-1, A), (C, A-1), (C, A)
+    auto mean_u = [&](int k) -> T {  // node (i, j + k)
+      const T s = ((lm[k] + lm[k + 1]) + cm[k]) + cm[k + 1];
+      return s * ((!IN && (j + k == 0 || j + k == ny)) ? (T)0.5 : (T)0.25);
+    };
+    T mu_lo = mean_u(0);
+    T rm_lo = MU[o - EW + 1];
+    T dlo = cu[0] - rr[0] + cv[0] - cv[1];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const T lu = X0[o + k * EW - 1], rw = X1[o + k * EW + 1], rm = MU[o + k * EW + 1];
+      const T d0 = cu[k + 1] - rr[k + 1] + cv[k + 1] - cv[k + 2];
+      const T dl = lu - cu[k + 1] + lv[k] - lv[k + 1];
+      const T m0 = cm[k + 1], xf = cu[k + 1], yf = cv[k + 1];
+      const T mu_hi = mean_u(k + 1);
+      const T sl = ((lm[k] + cm[k]) + lm[k + 1]) + cm[k + 1];   // node (i, j + k), v's order
+      const T sr = ((cm[k] + rm_lo) + cm[k + 1]) + rm;          // node (i + 1, j + k)
+      T mv_lo = sl * (T)0.25, mv_hi = sr * (T)0.25;
+      if (!IN) {
+        if (i == 0) mv_lo = sl * (T)0.5;
+        if (i == nx - 1) mv_hi = sr * (T)0.5;
+      }
+      T w = fma(m0, xf - rr[k + 1], (T)0);
+      w = fma(lm[k + 1], xf - lu, w);
+      if (IN) {
+        w = fma(mu_hi, xf - cu[k + 2], w);
+        w = fma(mu_lo, xf - cu[k], w);
+      } else {
+        w = j + k == ny - 1 ? fma((T)2 * mu_hi, xf, w) : fma(mu_hi, xf - cu[k + 2], w);
+        w = j + k == 0 ? fma((T)2 * mu_lo, xf, w) : fma(mu_lo, xf - cu[k], w);
+      }
+      T y = fma(m0, yf - cv[k + 2], (T)0);
+      y = fma(cm[k], yf - cv[k], y);
+      if (IN) {
+        y = fma(mv_hi, yf - rw, y);
+        y = fma(mv_lo, yf - lv[k], y);
+      } else {
+        y = i == nx - 1 ? fma((T)2 * mv_hi, yf, y) : fma(mv_hi, yf - rw, y);
+        y = i == 0 ? fma((T)2 * mv_lo, yf, y) : fma(mv_lo, yf - lv[k], y);
+      }
+      const T zu = bu[k] - wall_row<T>(w, ws, gd, g2, d0, dl);
+      const T zv = bv[k] - wall_row<T>(y, ws, gd, g2, d0, dlo);
+      ru[k] = this->act_u(k) ? zu : (T)0;
+      rv[k] = this->act_v(k) ? zv : (T)0;
+      dlo = d0;
+      mu_lo = mu_hi;
+      rm_lo = rm;
+    }
+    this->put(R0, R1, ru, rv);
+  }
+
+  template <bool ZERO, bool FIRST>
+  __device__ __forceinline__ void cheb(const LegArgs<T>& A, int s, const T* su, const T* sv) {
+    const T ca = A.ca[s], cb = A.cb[s];
+    const long long Q = vtab_plane(A.L);
+    const int P = A.L.P;
+    T cu[K + 2], cv[K + 1], rr[K + 1], lv[K + 1];
+    cu[0] = R0[o - EW];
+    cu[K + 1] = R0[o + K * EW];
+    cv[K] = R1[o + K * EW];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      cu[k + 1] = su[k];
+      cv[k] = sv[k];
+    }
+#pragma unroll
+    for (int k = 0; k <= K; ++k) {
+      rr[k] = R0[o + (k - 1) * EW + 1];
+      lv[k] = R1[o + k * EW - 1];
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      T zu = (T)0, zv = (T)0;
+      if (IN || (this->in_x() && j + k >= 0 && j + k < ny)) {
+        const T rw = R1[o + k * EW + 1];
+        const T* t = A.table + (j + k) * P + i;
+        auto at = [&](const T* q, int r, int c) { return GKB_LDG(q + sym4(r, c) * Q); };
+        // the patches of the nodes (i, j), (i, j + 1) and (i + 1, j)
+        const T t13 = at(t, 1, 3);
+        const T a1 = patch_dot<T>(at(t, 1, 0), at(t, 1, 1), at(t, 1, 2), t13, cu[k], cu[k + 1], lv[k], cv[k]);
+        const T a3 = patch_dot<T>(at(t, 3, 0), t13, at(t, 3, 2), at(t, 3, 3), cu[k], cu[k + 1], lv[k], cv[k]);
+        const T a0 = patch_dot<T>(at(t + P, 0, 0), at(t + P, 0, 1), at(t + P, 0, 2), at(t + P, 0, 3), cu[k + 1],
+                                  cu[k + 2], lv[k + 1], cv[k + 1]);
+        const T a2 = patch_dot<T>(at(t + 1, 2, 0), at(t + 1, 2, 1), at(t + 1, 2, 2), at(t + 1, 2, 3), rr[k], rr[k + 1],
+                                  cv[k], rw);
+        if (this->act_u(k)) zu = cheb_wall<T>(ca, a1 + a0, cb, FIRST ? (T)0 : du[k], FIRST);
+        if (this->act_v(k)) zv = cheb_wall<T>(ca, a3 + a2, cb, FIRST ? (T)0 : dv[k], FIRST);
+      }
+      du[k] = zu;
+      dv[k] = zv;
+      xu[k] = ZERO ? zu : xu[k] + zu;
+      xv[k] = ZERO ? zv : xv[k] + zv;
+    }
+    this->put(X0, X1, xu, xv);
   }
 };
 
@@ -620,13 +766,13 @@ __device__ __forceinline__ bool strip_inner(const Blk& B, const Lvl& L) {
   return leg_inner(L, ei, ei + G::EW - 1, ej, ej + G::EH - 1);
 }
 
-template <typename T, int DEG, class G, bool IN>
+template <typename T, int DEG, class G, class S>
 __device__ __forceinline__ void strip_down_in(const Blk& B, const LegArgs<T>& A, T* sm) {
   constexpr int EW = G::EW, K = G::K;
   const Lvl& L = A.L;
   const int P = L.P, ov = (int)L.off[1];
-  Strip<T, G, IN> g(L, (int)B.x * G::TW, (int)B.y * G::TH, sm);
-  g.load_fold(A);
+  S g(L, (int)B.x * G::TW, (int)B.y * G::TH, sm);
+  g.setup(A);
   g.load(A.b, P, ov, g.bu, g.bv);
   if (A.rd) {
 #pragma unroll
@@ -670,13 +816,13 @@ __device__ __forceinline__ void strip_down_in(const Blk& B, const LegArgs<T>& A,
   }
 }
 
-template <typename T, int DEG, class G, bool IN>
+template <typename T, int DEG, class G, class S>
 __device__ __forceinline__ void strip_up_in(const Blk& B, const LegArgs<T>& A, T* sm) {
   constexpr int EW = G::EW, K = G::K;
   const Lvl& L = A.L;
   const int P = L.P, ov = (int)L.off[1];
-  Strip<T, G, IN> g(L, (int)B.x * G::TW, (int)B.y * G::TH, sm);
-  g.load_fold(A);
+  S g(L, (int)B.x * G::TW, (int)B.y * G::TH, sm);
+  g.setup(A);
   g.load(A.xpre, P, ov, g.xu, g.xv);
   g.load(A.b, P, ov, g.bu, g.bv);
   g.put(g.X0, g.X1, g.xu, g.xv);
@@ -715,19 +861,20 @@ __device__ __forceinline__ void strip_up_in(const Blk& B, const LegArgs<T>& A, T
   g.store(A.xout, P, ov, g.xu, g.xv);
 }
 
-template <typename T, int DEG, class G>
-__device__ __forceinline__ void strip_down_body(const Blk& B, const LegArgs<T>& A, T* sm) {
-  if (strip_inner<G>(B, A.L)) strip_down_in<T, DEG, G, true>(B, A, sm);
-  else strip_down_in<T, DEG, G, false>(B, A, sm);
-}
-template <typename T, int DEG, class G>
-__device__ __forceinline__ void strip_up_body(const Blk& B, const LegArgs<T>& A, T* sm) {
-  if (strip_inner<G>(B, A.L)) strip_up_in<T, DEG, G, true>(B, A, sm);
-  else strip_up_in<T, DEG, G, false>(B, A, sm);
+template <typename T, int DEG, class G, bool DOWN, template <typename, class, bool> class S>
+__device__ __forceinline__ void strip_body(const Blk& B, const LegArgs<T>& A, T* sm) {
+  const bool in = strip_inner<G>(B, A.L);
+  if constexpr (DOWN) {
+    if (in) strip_down_in<T, DEG, G, S<T, G, true>>(B, A, sm);
+    else strip_down_in<T, DEG, G, S<T, G, false>>(B, A, sm);
+  } else {
+    if (in) strip_up_in<T, DEG, G, S<T, G, true>>(B, A, sm);
+    else strip_up_in<T, DEG, G, S<T, G, false>>(B, A, sm);
+  }
 }
 
 // how a level's legs are tiled; LEG_OFF: separate launches
-enum LegKind { LEG_OFF = 0, LEG_8, LEG_STRIP };
+enum LegKind { LEG_OFF = 0, LEG_8, LEG_STRIP, LEG_VAR };
 
 // geometry and body of one leg of kind KIND
 template <int DEG, int KIND, bool DOWN>
@@ -739,25 +886,30 @@ struct LegShape {
   static constexpr size_t smem() { return leg_smem<T, G>(); }
   static dim3 grid(const Lvl& L) { return dim3((L.n[0] + TW - 1) / TW, (L.n[1] + TH - 1) / TH, 1); }
 };
-template <int DEG, bool DOWN>
-struct LegShape<DEG, LEG_STRIP, DOWN> {
-  using G = StripTile<DEG, DOWN, 64, 32, 4>;
+template <class G_, bool VAR>
+struct StripShape {
+  using G = G_;
   static constexpr int NT = G::NT, TW = G::TW, TH = G::TH;
   template <typename T>
-  static constexpr size_t smem() { return G::template smem<T>(); }
+  static constexpr size_t smem() { return G::template smem<T>(VAR); }
   static dim3 grid(const Lvl& L) { return dim3((L.n[0] + TW - 1) / TW, (L.n[1] + TH - 1) / TH, 1); }
 };
+// 1024^2 mixed solves by tile: constant viscosity 64 x 32 61.8 ms, 32 x 32
+// 62.4, 64 x 64 77.0; variable 32 x 32 at two blocks per SM (128 registers)
+// 104 ms, at three (80) 108, 64 x 32 109. Eight rows per thread instead of
+// four: 69 ms (half the warps in flight).
+template <int DEG, bool DOWN>
+struct LegShape<DEG, LEG_STRIP, DOWN> : StripShape<StripTile<DEG, DOWN, 64, 32, 4>, false> {};
+template <int DEG, bool DOWN>
+struct LegShape<DEG, LEG_VAR, DOWN> : StripShape<StripTile<DEG, DOWN, 32, 32, 4>, true> {};
 
 template <typename T, int DEG, int KIND, bool DOWN>
 __device__ __forceinline__ void leg_body(const Blk& B, const LegArgs<T>& A, T* sm) {
   using S = LegShape<DEG, KIND, DOWN>;
-  if constexpr (KIND == LEG_STRIP) {
-    if constexpr (DOWN) strip_down_body<T, DEG, typename S::G>(B, A, sm);
-    else strip_up_body<T, DEG, typename S::G>(B, A, sm);
-  } else {
-    if constexpr (DOWN) leg_down_body<T, DEG, S::TILE, S::TILE>(B, A, sm);
-    else leg_up_body<T, DEG, S::TILE, S::TILE>(B, A, sm);
-  }
+  if constexpr (KIND == LEG_STRIP) strip_body<T, DEG, typename S::G, DOWN, Strip>(B, A, sm);
+  else if constexpr (KIND == LEG_VAR) strip_body<T, DEG, typename S::G, DOWN, StripVar>(B, A, sm);
+  else if constexpr (DOWN) leg_down_body<T, DEG, S::TILE, S::TILE>(B, A, sm);
+  else leg_up_body<T, DEG, S::TILE, S::TILE>(B, A, sm);
 }
 
 }  // namespace gkb
