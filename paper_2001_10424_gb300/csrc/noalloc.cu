@@ -13,6 +13,7 @@
 
 #include "../../include/gkb.h"
 #include "common.cuh"
+#include "compact.cuh"
 #include "ops.h"
 #include "solver.cuh"
 
@@ -83,10 +84,25 @@ extern "C" int gkb_apply_noalloc(const gkb_grid* grid, double mu0, double gamma,
   double* scratch = nullptr;
   int rc = noalloc_scratch(&scratch);
   if (rc != GKB_OK) return rc;
+  const bool in_cells = (op == GKB_OP_A), out_cells = (op == GKB_OP_AT);
+  const long long m = gkb::lvl_unknowns(L), nc = (long long)n3[0] * n3[1] * n3[2];
+  cudaStream_t s = (cudaStream_t)stream;
+  if (!gkb::overlap(x, in_cells ? nc : m, y, out_cells ? nc : m)) {
+    // straight between the compact vectors
+    try {
+      gkb::apply_compact(L, op, x, y, s);
+    } catch (const gkb::Error&) {
+      return GKB_ERR_CUDA;
+    }
+    if (cudaStreamSynchronize(s) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return GKB_ERR_CUDA;
+    }
+    return GKB_OK;
+  }
+  // in place: through the padded work arrays
   double* in = scratch;
   double* out = scratch + (size_t)GKB_NOALLOC_MAX_ELEMS;
-  cudaStream_t s = (cudaStream_t)stream;
-  const bool in_cells = (op == GKB_OP_A), out_cells = (op == GKB_OP_AT);
   // the previous call's contents remain in the array: clear the input's
   // padding, which the operator kernels read as zero
   if (cudaMemsetAsync(in, 0, (in_cells ? L.ncell : L.nvel) * sizeof(double), s) != cudaSuccess) {

@@ -16,6 +16,7 @@
 #include <cooperative_groups.h>
 
 #include "solver.cuh"
+#include "compact.cuh"
 #include "gkb_device.cuh"
 #include "lockstep.cuh"
 #include "prof.h"
@@ -84,38 +85,6 @@ template <> void set_nw<float>(Lvl& L, const float* w) { L.nw32 = w; L.nw64 = nu
 // ---------------------------------------------------------------------------
 // layout kernels (compact ordering <-> padded layout)
 // ---------------------------------------------------------------------------
-
-struct Compact {
-  int dim;
-  int lo[3][3];    // low corner of the active box of component c
-  int ext[3][3];   // extents of that box
-  long long base[3];
-  long long m;
-};
-
-static Compact make_compact(const Lvl& L) {
-  Compact c{};
-  c.dim = L.dim;
-  long long off = 0;
-  for (int comp = 0; comp < L.dim; ++comp) {
-    for (int a = 0; a < 3; ++a) {
-      if (a >= L.dim) { c.lo[comp][a] = 0; c.ext[comp][a] = 1; continue; }
-      if (a == comp) {
-        const int lo = L.nat[2 * a] ? 0 : 1;
-        const int hi = L.nat[2 * a + 1] ? L.n[a] : L.n[a] - 1;
-        c.lo[comp][a] = lo;
-        c.ext[comp][a] = hi - lo + 1;
-      } else {
-        c.lo[comp][a] = 0;
-        c.ext[comp][a] = L.n[a];
-      }
-    }
-    c.base[comp] = off;
-    off += (long long)c.ext[comp][0] * c.ext[comp][1] * c.ext[comp][2];
-  }
-  c.m = off;
-  return c;
-}
 
 __device__ __forceinline__ long long compact_to_padded(const Lvl& L, const Compact& c, long long t) {
   int comp = 0;
@@ -2119,6 +2088,18 @@ void Solver::apply(int op, const double* xin, double* yout) {
     GKB_CUDA(cudaMemcpyAsync(st_in, xin, nin * sizeof(double), cudaMemcpyHostToDevice, s));
     src = st_in;
   }
+  const bool ydev = is_device_ptr(yout);
+  double* dst = ydev ? yout : (out_cells ? stage_n.p : stage_m.p);
+  if (op < GKB_OP_W || op > GKB_OP_M) throw Error{GKB_ERR_INVALID_ARG, "unknown operator"};
+  // constant viscosity: straight between the compact vectors, unless the
+  // result would overwrite entries that other blocks still read
+  if (!mu64.p && !overlap(src, nin, dst, nout)) {
+    apply_compact(L, op, src, dst, s);
+    if (!ydev) GKB_CUDA(cudaMemcpyAsync(yout, dst, nout * sizeof(double), cudaMemcpyDeviceToHost, s));
+    GKB_CUDA(cudaStreamSynchronize(s));
+    GKB_CUDA(cudaGetLastError());
+    return;
+  }
   if (in_cells) {
     GKB_CUDA(cudaMemsetAsync(ctmp.p, 0, L.ncell * sizeof(double), s));
     { ProfScope ps_(GKB_KC_LAYOUT, s); k_pack_cell<double><<<lin_blocks(ncell), 256, 0, s>>>(L, src, ctmp.p); }
@@ -2131,10 +2112,7 @@ void Solver::apply(int op, const double* xin, double* yout) {
     case GKB_OP_M: Ops<double>::apply(L, 1, wtmp.p, t.p, s); break;
     case GKB_OP_A: Ops<double>::grad(L, ctmp.p, t.p, 1.0, s); break;
     case GKB_OP_AT: Ops<double>::negdiv(L, wtmp.p, q.p, 1.0, s); break;
-    default: throw Error{GKB_ERR_INVALID_ARG, "unknown operator"};
   }
-  const bool ydev = is_device_ptr(yout);
-  double* dst = ydev ? yout : (out_cells ? stage_n.p : stage_m.p);
   if (out_cells) { ProfScope ps_(GKB_KC_LAYOUT, s); k_unpack_cell<<<lin_blocks(ncell), 256, 0, s>>>(L, q.p, dst, 0.0); }
   else { ProfScope ps_(GKB_KC_LAYOUT, s); k_unpack_vel<<<lin_blocks(m), 256, 0, s>>>(L, cmp, t.p, dst); }
   if (!ydev) GKB_CUDA(cudaMemcpyAsync(yout, dst, nout * sizeof(double), cudaMemcpyDeviceToHost, s));
