@@ -977,6 +977,433 @@ __global__ void __launch_bounds__(SB) k_cg_cluster(Lvl L, const double* __restri
   }
 }
 
+// The same solve with every vector on chip, for problems whose padded length
+// fits: a block keeps x, r, p and s of its share in registers, every block
+// holds a copy of r (the entries its rows read) in shared memory and w of its
+// own share; the owner of an entry of r stores it into the blocks that read
+// it, the block that forms a row of w = M r stores it into the entry's owner.
+// An iteration is then a chain of FP64 latencies: about 60 cycles per
+// dependent operation, 840 per division, and a warp instruction keeps the
+// unit for 16 cycles of the SM however few lanes are on. Hence: rows with
+// their neighbours, link coefficients and cells looked up once (m_row's
+// operations in its order, but all differences and both divergences before
+// the chain of link sums); rows packed into as few warps as hold them; both
+// sums reduced together; a ninth warp for the scalars, which works out
+// 1 / gamma and 1 / alpha while the others update and multiply, so that two
+// of the recurrence's three divisions become three operations each. The
+// shares, the operations and the order of every sum are those of
+// k_cg_cluster, so the bits are too. 32 x 32 channel: 9.3 -> 5.1 us per
+// iteration.
+constexpr int CGS_E = 4;            // entries of its share per thread
+constexpr int CGS_F = 3;            // rows per thread
+constexpr int CGS_Q = 2;            // positions per thread
+constexpr int CGS_LEN = 12800;      // padded length at most (100 KB copy of r)
+constexpr int CGS_NT = SB + 32;     // eight warps and the scalars' warp
+constexpr int CGS_T = 4;            // blocks an entry is stored into, kept as addresses
+
+__device__ __forceinline__ unsigned remote_addr(const void* p, int rank) {
+  unsigned r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void remote_store(unsigned a, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+
+// a / b from y = 1 / b rounded to nearest (Markstein): q = a y is within an
+// ulp, its remainder a - b q is exact, and one correction rounds as the
+// division does. Outside the exponents where no term under- or overflows: the
+// division itself.
+__device__ __forceinline__ double div_by(double a, double b, double y) {
+  // biased exponents within 500 of 1 (integer tests: a comparison on the FP64
+  // unit costs as much as a multiply-add)
+  const unsigned ea = ((unsigned)__double2hiint(a) >> 20) & 0x7ff, eb = ((unsigned)__double2hiint(b) >> 20) & 0x7ff;
+  if (ea - 523u > 1000u || eb - 523u > 1000u) return a / b;
+  const double q = a * y;
+  return fma(fma(-b, q, a), y, q);
+}
+
+// one row of M, looked up once: face id, its links' neighbours (zero: a slot
+// that holds 0, for walls) and coefficients (0: no link), the cells on its
+// two sides (-1: outside) and their weights
+template <int DIM, bool VarMu>
+struct RowRef {
+  int id, comp, nb[2 * DIM], cell[2];
+  double k[2 * DIM], nw[VarMu ? 2 : 1];
+
+  template <int C>
+  __device__ void set(const Lvl& L, const int (&p)[3], int zero) {
+    comp = C;
+    id = (int)L.off[C] + (int)cix(L, p[0], p[1], p[2]);
+    const bool half = (p[C] == 0 && L.nat[2 * C]) || (p[C] == L.n[C] && L.nat[2 * C + 1]);
+    const double area = half ? 0.5 : 1.0;
+    int q[3] = {p[0], p[1], p[2]};
+    auto face = [&]() { return (int)L.off[C] + (int)cix(L, q[0], q[1], q[2]); };
+    k[0] = k[1] = 0.0;
+    nb[0] = nb[1] = zero;
+    if (p[C] < L.n[C]) {
+      k[0] = cell_mu<double, VarMu>(L, p[0], p[1], p[2]);
+      q[C] = p[C] + 1;
+      nb[0] = face();
+    }
+    if (p[C] > 0) {
+      q[C] = p[C] - 1;
+      k[1] = cell_mu<double, VarMu>(L, q[0], q[1], q[2]);
+      nb[1] = face();
+    }
+    q[C] = p[C];
+    int l = 2;
+#pragma unroll
+    for (int A = 0; A < DIM; ++A) {
+      if (A == C) continue;
+#pragma unroll
+      for (int hi = 1; hi >= 0; --hi) {  // the link across A-coordinate p[A] + 1, then p[A]
+        const int af = p[A] + hi;
+        double mu;
+        if (A == 0) mu = edge_mu<double, VarMu, C, C == 0 ? 1 : 0>(L, p, af);
+        else if (A == 1) mu = edge_mu<double, VarMu, C, C == 1 ? 0 : 1>(L, p, af);
+        else mu = edge_mu<double, VarMu, C, C == 2 ? 0 : 2>(L, p, af);
+        const bool inside = hi ? p[A] + 1 < L.n[A] : p[A] > 0;
+        nb[l] = zero;
+        k[l] = 0.0;
+        if (inside) {
+          q[A] = hi ? p[A] + 1 : p[A] - 1;
+          nb[l] = face();
+          q[A] = p[A];
+          k[l] = area * mu;
+        } else if (!L.nat[2 * A + hi]) {
+          k[l] = 2.0 * area * mu;
+        }
+        ++l;
+      }
+    }
+    for (int s = 0; s < 2; ++s) {
+      q[C] = p[C] - s;
+      const bool in = cell_in(L, q[0], q[1], q[2]);
+      cell[s] = in ? (int)cix(L, q[0], q[1], q[2]) : -1;
+      if (VarMu) nw[VarMu ? s : 0] = in ? cell_nw<double, VarMu>(L, cix(L, q[0], q[1], q[2])) : 1.0;
+    }
+  }
+
+  __device__ __forceinline__ double row(const Lvl& L, const double* r) const {
+    const double xf = r[id];
+    double d[2 * DIM], c[2];
+#pragma unroll
+    for (int l = 0; l < 2 * DIM; ++l) d[l] = xf - r[nb[l]];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const int at = cell[s] < 0 ? 0 : cell[s];
+      const double* u = r + at;
+      const double* v = r + L.off[1] + at;
+      double t = u[0] - u[1] + v[0] - v[L.P];
+      if (DIM == 3) {
+        const double* w = r + L.off[2] + at;
+        t += w[0] - w[L.S];
+      }
+      if (VarMu) t *= nw[VarMu ? s : 0];
+      c[s] = cell[s] < 0 ? 0.0 : t;
+    }
+    double acc = fma(k[0], d[0], 0.0);
+#pragma unroll
+    for (int l = 1; l < 2 * DIM; ++l) acc = fma(k[l], d[l], acc);
+    const double wv = acc * L.wscale;
+    if (!L.has_gd) return wv;
+    return wv + L.g2 * (c[0] - c[1]);
+  }
+};
+
+template <int DIM, bool VarMu>
+__global__ void __launch_bounds__(CGS_NT) k_cg_cluster_sm(const __grid_constant__ Lvl L, const double* __restrict__ f,
+                                                           double* __restrict__ x, CgState* c, double tol2, int maxit) {
+  namespace cgx = cooperative_groups;
+  cgx::cluster_group cl = cgx::this_cluster();
+  extern __shared__ __align__(16) double cg_sm[];
+  __shared__ double sh[2][8];
+  __shared__ double slots[2][16][2];
+  __shared__ double s_alpha, s_beta;
+  __shared__ int s_stop, s_faces;
+  int phase = 0;
+  const int rank = (int)cl.block_rank(), nb = (int)cl.num_blocks(), tid = threadIdx.x;
+  const int lane = tid & 31, warp = tid >> 5;
+  const bool ctl = warp == SB / 32;  // the scalars' warp
+  const int len = (int)L.nvel;
+  const int nx = L.n[0] + 1, ny = L.n[1] + 1, nz = (DIM == 3) ? L.n[2] + 1 : 1;
+  const int npos = nx * ny * nz;
+  const int vch = (len + nb - 1) / nb, pch = (npos + nb - 1) / nb;
+  const int v0 = rank * vch, v1 = min(len, v0 + vch);
+  const int p0 = rank * pch, p1 = min(npos, p0 + pch);
+  double* rf = cg_sm;            // r, indexed like the padded array, and a zero
+  double* wo = rf + len + 1;     // w of this block's share
+  double* wl = wo + vch;         // w of this block's rows, [component][position - p0]
+  int* faces = (int*)(wl + DIM * pch);  // DIM (position - p0) + component of the block's active faces
+  // this thread's entries and the blocks whose positions read each of them
+  // (rows reach one position in every axis)
+  double xr[CGS_E], rr_[CGS_E], pr[CGS_E], sr[CGS_E];
+  int lo[CGS_E], hi[CGS_E];
+  unsigned to[CGS_E][CGS_T];
+  const int reach = (DIM == 3 ? nx * ny : 0) + nx + 1;
+  double ff = 0.0;
+  bool live = false;
+#pragma unroll
+  for (int e = 0; e < CGS_E; ++e) {
+    const int t = v0 + tid + e * SB;
+    xr[e] = rr_[e] = pr[e] = sr[e] = 0.0;
+    lo[e] = 1;
+    hi[e] = 0;
+    if (!ctl && t < v1) {
+      const double ft = f[t];
+      rr_[e] = ft;
+      ff += ft * ft;
+      const int comp = (DIM == 3 && t >= L.off[2]) ? 2 : t >= L.off[1] ? 1 : 0;
+      const int q = t - (int)L.off[comp], k = q / (int)L.S, j = (q - k * (int)L.S) / L.P, i = q - k * (int)L.S - j * L.P;
+      if (i < nx) {
+        const int pos = (k * ny + j) * nx + i;
+        lo[e] = max(0, pos - reach) / pch;
+        hi[e] = min(npos - 1, pos + reach) / pch;
+        live = true;
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < CGS_T; ++b) to[e][b] = lo[e] + b <= hi[e] ? remote_addr(rf + t, lo[e] + b) : 0u;
+  }
+  // a warp whose entries are all padding (0) skips the updates and its sum
+  const bool wlive = __any_sync(0xffffffffu, live);
+  const bool wpos = !ctl && warp * 32 < p1 - p0;  // this warp owns positions
+  for (int t = tid; t <= len; t += CGS_NT) rf[t] = 0.0;
+  for (int t = tid; t < vch; t += CGS_NT) wo[t] = 0.0;
+  for (int t = tid; t < DIM * pch; t += CGS_NT) wl[t] = 0.0;
+  auto where = [&](int q, int (&p)[3]) {  // position p0 + q
+    const int u = (p0 + q) / nx;
+    p[0] = p0 + q - u * nx;
+    p[1] = u % ny;
+    p[2] = u / ny;
+  };
+  auto active = [&](int comp, const int (&p)[3]) {
+    return comp == 0 ? face_active<0>(L, p[0], p[1], p[2])
+                     : comp == 1 ? face_active<1>(L, p[0], p[1], p[2]) : face_active<2>(L, p[0], p[1], p[2]);
+  };
+  if (warp == 0) {  // the active faces, in order
+    int n = 0;
+    for (int comp = 0; comp < DIM; ++comp)
+      for (int q0 = 0; q0 < p1 - p0; q0 += 32) {
+        int p[3];
+        where(q0 + lane, p);
+        const bool on = q0 + lane < p1 - p0 && active(comp, p);
+        const unsigned m = __ballot_sync(0xffffffffu, on);
+        if (on) faces[n + __popc(m & ((1u << lane) - 1))] = DIM * (q0 + lane) + comp;
+        n += __popc(m);
+      }
+    if (lane == 0) s_faces = n;
+  }
+  cl.sync();  // every block's copy is cleared, its faces listed
+  const int nf = s_faces;
+  RowRef<DIM, VarMu> rows[CGS_F];
+  unsigned w_to[CGS_F];
+  int w_at[CGS_F];
+#pragma unroll
+  for (int e = 0; e < CGS_F; ++e) {
+    w_at[e] = -1;
+    const int t = tid + e * SB;
+    if (!ctl && t < nf) {
+      const int q = faces[t] / DIM, comp = faces[t] - DIM * q;
+      int p[3];
+      where(q, p);
+      if (comp == 0) rows[e].template set<0>(L, p, len);
+      else if (comp == 1) rows[e].template set<1>(L, p, len);
+      else if constexpr (DIM == 3) rows[e].template set<2>(L, p, len);
+      w_at[e] = comp * pch + q;
+      w_to[e] = remote_addr(wo + rows[e].id % vch, rows[e].id / vch);
+    }
+  }
+  int pos_id[CGS_Q][DIM];  // flat index of this thread's positions' active faces, or -1
+#pragma unroll
+  for (int e = 0; e < CGS_Q; ++e) {
+    const int q = tid + e * SB;
+    int p[3];
+    where(q, p);
+#pragma unroll
+    for (int comp = 0; comp < DIM; ++comp)
+      pos_id[e][comp] = (!ctl && q < p1 - p0 && active(comp, p)) ? (int)L.off[comp] + (int)cix(L, p[0], p[1], p[2]) : -1;
+  }
+  auto push = [&]() {
+#pragma unroll
+    for (int e = 0; e < CGS_E; ++e) {
+#pragma unroll
+      for (int b = 0; b < CGS_T; ++b)
+        if (lo[e] + b <= hi[e]) remote_store(to[e][b], rr_[e]);
+      for (int b = lo[e] + CGS_T; b <= hi[e]; ++b) remote_store(remote_addr(rf + v0 + tid + e * SB, b), rr_[e]);
+    }
+  };
+  // w = M r on this block's faces, stored at its owners; then (r, w) over its
+  // positions
+  auto apply = [&]() -> double {
+#pragma unroll
+    for (int e = 0; e < CGS_F; ++e)
+      if (w_at[e] >= 0) {
+        const double v = rows[e].row(L, rf);
+        wl[w_at[e]] = v;
+        remote_store(w_to[e], v);
+      }
+    __syncthreads();
+    double pq = 0.0;
+#pragma unroll
+    for (int e = 0; e < CGS_Q; ++e)
+#pragma unroll
+      for (int comp = 0; comp < DIM; ++comp)
+        if (pos_id[e][comp] >= 0) pq += rf[pos_id[e][comp]] * wl[comp * pch + tid + e * SB];
+    return pq;
+  };
+  // the cluster's sums of (a, b), each block's stored into every block before
+  // the barrier; valid in the scalars' warp, lane 0 (the widths leave out only
+  // additions of 0)
+  auto sums = [&](double a, double b, double& ta, double& tb) {
+    if (wlive || wpos) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_down_sync(0xffffffffu, a, o);
+        b += __shfl_down_sync(0xffffffffu, b, o);
+      }
+    }
+    if (!ctl && lane == 0) {
+      sh[0][warp] = a;
+      sh[1][warp] = b;
+    }
+    __syncthreads();
+    if (ctl) {
+      a = lane < 8 ? sh[0][lane] : 0.0;
+      b = lane < 8 ? sh[1][lane] : 0.0;
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) {
+        a += __shfl_down_sync(0xffffffffu, a, o);
+        b += __shfl_down_sync(0xffffffffu, b, o);
+      }
+      a = __shfl_sync(0xffffffffu, a, 0);
+      b = __shfl_sync(0xffffffffu, b, 0);
+      if (lane < nb) {
+        const unsigned d = remote_addr(&slots[phase][rank][0], lane);
+        remote_store(d, a);
+        remote_store(d + 8, b);
+      }
+    }
+    cl.sync();
+    if (ctl) {
+      a = lane < nb ? slots[phase][lane][0] : 0.0;
+      b = lane < nb ? slots[phase][lane][1] : 0.0;
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) {
+        a += __shfl_down_sync(0xffffffffu, a, o);
+        b += __shfl_down_sync(0xffffffffu, b, o);
+      }
+      ta = a;
+      tb = b;
+    }
+    phase ^= 1;
+  };
+  push();
+  cl.sync();  // r complete
+  // the recurrence's scalars live in the scalars' warp of every block (the
+  // same values), with the reciprocals of gamma and alpha
+  double gamma = 0.0, delta = 0.0, gamma_prev = 0.0, alpha = 0.0, y_gamma = 0.0, y_alpha = 0.0, stop_at = 0.0;
+  int it = 0, status = ST_OK;
+  auto step = [&]() {  // the next alpha and beta, or the end
+    int stop = 0;
+    double beta = 0.0, den = delta;
+    if (it > 0) {  // beta = gamma / gamma_prev, den = delta - beta gamma / alpha
+      beta = div_by(gamma, gamma_prev, y_gamma);
+      den = delta - div_by(beta * gamma, alpha, y_alpha);
+    }
+    if (!(den > 0.0)) {
+      status = isfinite(den) ? ST_NOT_SPD : ST_NAN;
+      stop = 1;
+    } else {
+      alpha = gamma / den;
+    }
+    s_alpha = alpha;
+    s_beta = beta;
+    s_stop = stop;
+  };
+  {
+    const double pq = apply();
+    sums(ff, pq, gamma, delta);  // (r, r), (M r, r)
+  }
+  if (ctl && lane == 0) {
+    ff = gamma;
+    stop_at = tol2 * ff;
+    if (!isfinite(ff) || !isfinite(delta)) status = ST_NAN;
+    if (ff == 0.0 || status != ST_OK) s_stop = 1;
+    else step();
+  }
+  __syncthreads();
+  while (!s_stop) {
+    double rr = 0.0;
+    if (wlive) {
+      const double al = s_alpha, be = s_beta;
+#pragma unroll
+      for (int e = 0; e < CGS_E; ++e) {
+        if (v0 + tid + e * SB < v1) {
+          const double pt = rr_[e] + be * pr[e];
+          const double st = wo[tid + e * SB] + be * sr[e];
+          pr[e] = pt;
+          sr[e] = st;
+          const double rt = rr_[e] - al * st;
+          rr_[e] = rt;
+          rr += rt * rt;
+        }
+      }
+      push();
+      cl.barrier_arrive();
+#pragma unroll
+      for (int e = 0; e < CGS_E; ++e)
+        if (v0 + tid + e * SB < v1) xr[e] += al * pr[e];
+    } else {
+      cl.barrier_arrive();
+      if (ctl && lane == 0) {  // for the next iteration's quotients
+        y_gamma = 1.0 / gamma;
+        y_alpha = 1.0 / alpha;
+      }
+      __syncwarp();
+    }
+    cl.barrier_wait();  // r complete before the product reads neighbours
+    const double pq = apply();
+    double g = 0.0, d = 0.0;
+    sums(rr, pq, g, d);
+    if (ctl && lane == 0) {
+      ++it;
+      gamma_prev = gamma;
+      gamma = g;
+      delta = d;
+      if (!isfinite(gamma) || !isfinite(delta)) {
+        status = ST_NAN;
+        s_stop = 1;
+      } else if (gamma <= stop_at) {
+        s_stop = 1;
+      } else if (it >= maxit) {
+        status = ST_INNER_NOT_CONVERGED;
+        s_stop = 1;
+      } else {
+        step();
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int e = 0; e < CGS_E; ++e)
+    if (!ctl && v0 + tid + e * SB < v1) x[v0 + tid + e * SB] = xr[e];
+  if (rank == 0 && ctl && lane == 0) {
+    c->ff = ff;
+    c->rr = gamma;
+    c->it = it;
+    c->total_it += it;
+    c->solves += 1;
+    c->status = status;
+    c->done = 1;
+    c->graph_iters = 0;
+    c->fb_iters = 0;
+    c->fallback = 0;
+  }
+  cl.sync();  // no block leaves while another may still store into it
+}
+
 // record an inner solve in the GKB state: status, iterations, history
 __global__ void k_note_inner(GkbState* S, const CgState* c) {
   const int idx = S->inner_solves;
@@ -1512,17 +1939,17 @@ bool Solver::small_cg() const {
   return opt.inner == GKB_INNER_CG && opt.precision == GKB_PREC_FP64 && L64.nvel <= (1LL << 15);
 }
 
-// cluster size for k_cg_cluster: 16 blocks where the device allows it, else
-// 8 (decided once per device and kernel)
-static int cg_cluster_size(bool var_mu) {
+// cluster size of the single-kernel CG: 16 blocks where the device allows it,
+// else 8 (decided once per device and kernel; smem: its dynamic shared memory)
+static int cg_cluster_size(const void* fn, int slot, size_t smem, int threads) {
   static std::mutex mtx;
   static std::map<int, int> cached;
   int dev = 0;
   GKB_CUDA(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lock(mtx);
-  int& cs = cached[2 * dev + (var_mu ? 1 : 0)];
+  int& cs = cached[6 * dev + slot];
   if (cs) return cs;
-  const void* fn = var_mu ? (const void*)k_cg_cluster<true> : (const void*)k_cg_cluster<false>;
+  if (smem) GKB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   cs = 8;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
     cudaLaunchConfig_t cfg = {};
@@ -1532,7 +1959,8 @@ static int cg_cluster_size(bool var_mu) {
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(16);
-    cfg.blockDim = dim3(SB);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
@@ -1547,7 +1975,20 @@ void Solver::launch_cg_block(const double* fpad, double* xpad, cudaStream_t s) {
   ProfScope ps_(GKB_KC_APPLY, s, 0);  // unknowns counted per iteration in finish()
   const double tol2 = opt.tol_inner * opt.tol_inner;
   const bool var = L64.mu64 != nullptr;
-  const int cs = cg_cluster_size(var);
+  // every vector on chip where a block's copy of r and the threads' entries
+  // have room
+  constexpr size_t max_sm = 190 * 1024;
+  const bool d3 = L64.dim == 3;
+  auto sm_fn = d3 ? (var ? k_cg_cluster_sm<3, true> : k_cg_cluster_sm<3, false>)
+                  : (var ? k_cg_cluster_sm<2, true> : k_cg_cluster_sm<2, false>);
+  int cs = cg_cluster_size((const void*)sm_fn, 2 + (var ? 1 : 0) + (d3 ? 2 : 0), max_sm, CGS_NT);
+  const long long npos = (L64.n[0] + 1LL) * (L64.n[1] + 1) * (d3 ? L64.n[2] + 1 : 1);
+  const long long vch = (L64.nvel + cs - 1) / cs, pch = (npos + cs - 1) / cs, dim = L64.dim;
+  const size_t sm = (size_t)(L64.nvel + 1 + vch + dim * pch) * sizeof(double) + (size_t)(dim * pch) * sizeof(int);
+  const bool chip = L64.nvel <= CGS_LEN && vch <= CGS_E * SB && pch <= CGS_Q * SB && dim * pch <= CGS_F * SB &&
+                    sm <= max_sm && !L64.sym;
+  const void* fn = var ? (const void*)k_cg_cluster<true> : (const void*)k_cg_cluster<false>;
+  if (!chip) cs = cg_cluster_size(fn, var ? 1 : 0, 0, SB);
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1559,12 +2000,17 @@ void Solver::launch_cg_block(const double* fpad, double* xpad, cudaStream_t s) {
   cfg.stream = s;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (var)
+  if (chip) {
+    cfg.dynamicSmemBytes = sm;
+    cfg.blockDim = dim3(CGS_NT);
+    GKB_CUDA(cudaLaunchKernelEx(&cfg, sm_fn, L64, fpad, xpad, cg_dev, tol2, opt.maxit_inner));
+  } else if (var) {
     GKB_CUDA(cudaLaunchKernelEx(&cfg, k_cg_cluster<true>, L64, fpad, xpad, c.r.p, c.p.p, c.q.p, c.z.p, cg_dev,
                                 tol2, opt.maxit_inner));
-  else
+  } else {
     GKB_CUDA(cudaLaunchKernelEx(&cfg, k_cg_cluster<false>, L64, fpad, xpad, c.r.p, c.p.p, c.q.p, c.z.p, cg_dev,
                                 tol2, opt.maxit_inner));
+  }
 }
 
 int Solver::inner_solve(const double* fpad, double* xpad) {
