@@ -181,7 +181,7 @@ void Ops<KT>::prolong(const Lvl& Lf, const Lvl& Lc, const KT* xc, KT* xf, KT* sl
   }
   { ProfScope ps_(GKB_KC_PROLONG, s, 0); k_slopes3d<KT><<<face_grid(Lc), dim3(BX, BY), 0, s>>>(Lc, xc, slopes); }
   ProfScope ps_(GKB_KC_PROLONG, s, lvl_unknowns(Lf));
-  k_prolong_flux3d<KT><<<face_grid(Lf), dim3(BX, BY), 0, s>>>(Lf, Lc, xc, slopes, xf);
+  k_prolong_flux3d<KT><<<cell_grid(Lc), dim3(BX, BY), 0, s>>>(Lf, Lc, xc, slopes, xf);
 }
 
 template <>

@@ -1,4 +1,5 @@
 // legs.cu - launches of the fused V-cycle legs (legs.cuh).
+#include <climits>
 #include "legs.cuh"
 #include "solver.cuh"
 
@@ -85,6 +86,7 @@ void gmg_leg_plan(Gmg<T>& G) {
     auto& V = G.lev[l];
     V.leg = LEG_OFF;
     if (l + 1 == G.lev.size() || V.L.dim != 2 || !V.L.fast || G.degree > LEG_MAX_DEG) continue;
+    if (V.L.nvel > INT_MAX) continue;  // the legs index with 32 bits
     if (!V.fold_in.empty() && cheb2_level(V.L)) V.leg = leg_kind<T>(V.L);
     // FP32 variable viscosity with N = n I and the Laplacian form
     else if (sizeof(T) == 4 && V.L.mu32 && !V.L.nw32 && !V.L.sym) V.leg = LEG_VAR;
