@@ -373,7 +373,19 @@ __global__ void __launch_bounds__(BX* BY) k_mac_tile(Lvl L, int wonly, const T* 
 // link-by-link row. Both use the operations and roundings of k_mac_tile, so
 // the values are bit for bit its (the dot sums in another order).
 // ---------------------------------------------------------------------------
-constexpr int MAC3_KZ = 16;
+// planes a box block walks: 16, halved while the level would leave the chip
+// below three blocks an SM (a walk is a chain of loads, one plane's latency
+// after the other; every block loads two planes more than it writes). 64^3:
+// smoother 16.2 -> 14.1 us, residual 15.5 -> 14.6 us; 160^3 keeps 16
+__host__ __device__ __forceinline__ int walk_kz(const Lvl& L, int margin, int gx, int gy) {
+  const int nz = L.n[2] > margin ? L.n[2] - margin : 0;
+  int kz = 16;
+  while (kz > 2 && gx * gy * ((nz + kz - 1) / kz) < 456) kz >>= 1;
+  return kz;
+}
+__host__ __device__ __forceinline__ int mac3_kz(const Lvl& L) {
+  return walk_kz(L, 2, (L.n[0] - 2 + BX - 1) / BX, (L.n[1] - 2 + BY - 1) / BY);
+}
 
 // levels that take the split kernels (smaller ones stay with k_mac_tile)
 inline bool mac3_level(const Lvl& L) {
@@ -415,7 +427,7 @@ __device__ __forceinline__ void shell_ijk(const Lvl& L, int lo, int hi, long lon
 // the shell of the operator's box [1, n-2]
 __host__ __device__ __forceinline__ long long mac3_shell_count(const Lvl& L) { return shell_count(L, 1, 2); }
 // z extent of the box part of the launch; z slices beyond it are the shell's
-__host__ __device__ __forceinline__ int mac3_box_z(const Lvl& L) { return (L.n[2] - 2 + MAC3_KZ - 1) / MAC3_KZ; }
+__host__ __device__ __forceinline__ int mac3_box_z(const Lvl& L) { return L.n[2] > 2 ? (L.n[2] - 2 + mac3_kz(L) - 1) / mac3_kz(L) : 0; }
 // one launch: the box's blocks, then enough z slices of blocks for one
 // thread per shell position
 inline dim3 mac3_grid(const Lvl& L) {
@@ -436,9 +448,9 @@ __device__ __forceinline__ double mac3_box_body(const Blk& B, const Lvl& L, int 
   __shared__ T Xt[4][3][TH][TW];                  // [plane slot][component][row][col]: position (i0-1+col, j0-1+row)
   __shared__ T Dv[SD ? 3 : 1][BY + 1][BX + 1];     // [cell plane slot][row][col]: cell (i0-1+col, j0-1+row)
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * BX + tx;
-  const int i0 = 1 + (int)B.x * BX, j0 = 1 + (int)B.y * BY, k0 = 1 + (int)B.z * MAC3_KZ;
+  const int i0 = 1 + (int)B.x * BX, j0 = 1 + (int)B.y * BY, k0 = 1 + (int)B.z * mac3_kz(L);
   const int i = i0 + tx, j = j0 + ty;
-  const int kend = min(k0 + MAC3_KZ, L.n[2] - 1);  // planes k0 .. kend-1 (uniform over the block)
+  const int kend = min(k0 + mac3_kz(L), L.n[2] - 1);  // planes k0 .. kend-1 (uniform over the block)
   const bool mine = i <= L.n[0] - 2 && j <= L.n[1] - 2;
   const bool gd = L.has_gd && !wonly;
   auto slot = [](int k) { return k & 3; };   // k >= 0
@@ -1359,12 +1371,14 @@ __global__ void __launch_bounds__(BX* BY) k_cheb3(Lvl L, const T* GKB_RESTRICT r
 // the same launch) takes the class table one thread per position. The same
 // operations as k_cheb3 for every face.
 // ---------------------------------------------------------------------------
-constexpr int CHEB3S_KZ = 16;
+__host__ __device__ __forceinline__ int cheb3s_kz(const Lvl& L) {
+  return walk_kz(L, 5, (L.n[0] - 5 + BX - 1) / BX, (L.n[1] - 5 + BY - 1) / BY);
+}
 
 inline bool cheb3s_level(const Lvl& L) {
   return L.dim == 3 && L.n[0] >= 16 && L.n[1] >= 16 && L.n[2] >= 16;
 }
-__host__ __device__ __forceinline__ int cheb3s_box_z(const Lvl& L) { return (L.n[2] - 5 + CHEB3S_KZ - 1) / CHEB3S_KZ; }
+__host__ __device__ __forceinline__ int cheb3s_box_z(const Lvl& L) { return L.n[2] > 5 ? (L.n[2] - 5 + cheb3s_kz(L) - 1) / cheb3s_kz(L) : 0; }
 inline dim3 cheb3s_grid(const Lvl& L) {
   const unsigned gx = (L.n[0] - 5 + BX - 1) / BX, gy = (L.n[1] - 5 + BY - 1) / BY;
   const long long per_slice = (long long)gx * gy * BX * BY;
@@ -1414,9 +1428,9 @@ __device__ __forceinline__ void cheb3s_box_body(const Blk& B, const Lvl& L, cons
   constexpr int TW = BX + 2, TH = BY + 2;
   __shared__ T Rt[4][3][TH][TW];   // [plane slot][component][row][col]: position (i0-1+col, j0-1+row); four slots: one barrier a plane
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * BX + tx;
-  const int i0 = 3 + (int)B.x * BX, j0 = 3 + (int)B.y * BY, k0 = 3 + (int)B.z * CHEB3S_KZ;
+  const int i0 = 3 + (int)B.x * BX, j0 = 3 + (int)B.y * BY, k0 = 3 + (int)B.z * cheb3s_kz(L);
   const int i = i0 + tx, j = j0 + ty;
-  const int kend = min(k0 + CHEB3S_KZ, L.n[2] - 2);  // planes k0 .. kend-1 (uniform over the block)
+  const int kend = min(k0 + cheb3s_kz(L), L.n[2] - 2);  // planes k0 .. kend-1 (uniform over the block)
   const bool mine = i <= L.n[0] - 3 && j <= L.n[1] - 3;
   auto slot = [](int k) { return k & 3; };
   // tile entries as in k_mac3's box (planes k0-1 .. kend lie in [2, n-2])
