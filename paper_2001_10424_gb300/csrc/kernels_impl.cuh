@@ -353,6 +353,20 @@ __device__ __forceinline__ void mac_tile_body(const Blk& B, const Lvl& L, int wo
   }
 }
 
+// the residual of a launch that is mostly skipped: at most eight blocks an SM
+// walk the grid of k_mac_tile, so that a skipped launch costs no more blocks
+template <typename T, bool VarMu>
+__global__ void __launch_bounds__(BX* BY) k_residual_if(Lvl L, dim3 g, const T* GKB_RESTRICT x, const T* GKB_RESTRICT b,
+                                                        T* GKB_RESTRICT r, const int* pred) {
+  if (!*pred) return;
+  const unsigned gxy = g.x * g.y;
+  for (unsigned t = blockIdx.x; t < gxy * g.z; t += gridDim.x) {
+    const unsigned z = t / gxy, q = t - z * gxy;
+    __syncthreads();  // the tiles of the block before
+    mac_tile_body<T, VarMu, 0, false>(Blk{q % g.x, q / g.x, z, g.x, g.y, g.z}, L, 0, x, b, r, RedBuf{nullptr, nullptr}, 0, nullptr, nullptr);
+  }
+}
+
 template <typename T, bool VarMu, int MODE, bool DOT>
 __global__ void __launch_bounds__(BX* BY) k_mac_tile(Lvl L, int wonly, const T* GKB_RESTRICT x, const T* GKB_RESTRICT b,
                                                      T* GKB_RESTRICT y, RedBuf red, int fin, void* st, const int* pred) {
@@ -385,6 +399,220 @@ __host__ __device__ __forceinline__ int walk_kz(const Lvl& L, int margin, int gx
 }
 __host__ __device__ __forceinline__ int mac3_kz(const Lvl& L) {
   return walk_kz(L, 2, (L.n[0] - 2 + BX - 1) / BX, (L.n[1] - 2 + BY - 1) / BY);
+}
+
+// ---- 2D operator with its inner product in column strips --------------------
+// y = M x and x . y of a large 2D level. The tile kernel spends its time on
+// the sum, not on the rows: 4257 blocks of 1024^2 each end in a block sum, a
+// fence and a ticket, and both factors of every product are converted on the
+// FP64 unit. Here a warp takes 60 columns x 1 to 8 rows, two columns a lane,
+// up the rows with three rows of loads in flight; neighbours come from the
+// next lane or the next register row, and a block sums eight strips at
+// once. Positions within one of a side are the shell: one
+// thread each, the general rows. Values are the tile kernel's, bit for bit.
+constexpr int MAC2_W = 60;
+// Levels it takes. FP32: 512^2 18.9 -> 14.6 us, 1024^2 41.3 -> 23.9 us, 2048^2
+// 131 -> 49.8 us (variable viscosity, 1024^2: 53.6 -> 27.5 us), but 256^2 12.5
+// -> 13.6 us; FP64: 512^2 31.1 -> 22.5 us, 1024^2 72.1 -> 56.2 us, 2048^2 293
+// -> 198 us, but 384^2 22.6 -> 24.4 us. 1024^2 is held by the FP64 unit in
+// both (FP32: its two products per position and their block sums)
+template <typename T> struct Mac2 { static constexpr long long MIN = 1LL << (sizeof(T) == 4 ? 17 : 18); };
+// rows a warp walks: as many (to 8) as leave 12 warps an SM. Fewer warps
+// leave latency exposed, more blocks cost sums (512^2 FP32 with 8, 12, 24 warps
+// an SM: 14.6, 14.6, 18.4 us; 768^2 21.8, 17.7, 21.0 us)
+__host__ __device__ __forceinline__ int mac2_ky(const Lvl& L) {
+  const long long w = (long long)((L.n[0] - 1 + MAC2_W - 1) / MAC2_W) * (L.n[1] - 2), fill = 152 * 12;
+  return w >= 8 * fill ? 8 : w >= 4 * fill ? 4 : w >= 2 * fill ? 2 : 1;
+}
+
+// constant viscosity, or cell viscosities with N = n I and the Laplacian form
+template <typename T>
+__host__ __device__ __forceinline__ bool mac2_level(const Lvl& L) {
+  const bool plain = sizeof(T) == 4 ? !L.nw32 && !L.em32 : !L.nw64 && !L.em64;
+  return L.dim == 2 && L.fast && L.n[0] * (long long)L.n[1] >= Mac2<T>::MIN && L.n[0] >= 48 && L.n[1] >= 8 && !L.sym && plain;
+}
+__host__ __device__ __forceinline__ int mac2_box_y(const Lvl& L) {
+  const int rows = BY * mac2_ky(L);
+  return (L.n[1] - 2 + rows - 1) / rows;
+}
+// the box's rows of blocks, then enough of them for one thread per shell position
+template <typename T>
+inline dim3 mac2_grid(const Lvl& L) {
+  const unsigned gx = (L.n[0] - 1 + MAC2_W - 1) / MAC2_W;
+  const long long shell = 3LL * (L.n[0] + 1) + 3LL * (L.n[1] - 2), per_row = (long long)gx * BX * BY;
+  return dim3(gx, mac2_box_y(L) + (unsigned)((shell + per_row - 1) / per_row));
+}
+
+template <typename T>
+struct alignas(2 * sizeof(T)) Two { T a, b; };
+
+template <typename T, bool VarMu>
+__device__ __forceinline__ double mac2_box_body(const Blk& B, const Lvl& L, int wonly, const T* GKB_RESTRICT x,
+                                                T* GKB_RESTRICT y) {
+  const int ky = mac2_ky(L);
+  const int lane = threadIdx.x, ia = (int)B.x * MAC2_W - 2 + 2 * lane;  // this lane's columns ia, ia + 1
+  const int j0 = 1 + ((int)B.y * BY + threadIdx.y) * ky;
+  if (j0 > L.n[1] - 2) return 0.0;  // whole warps
+  const bool gd = L.has_gd && !wonly, in = ia >= 0 && ia < L.P;
+  const T* mu = MuPtr<T>::get(L);
+  struct Row { Two<T> u, v, m; };
+  const T* xp = x + ia;
+  const T* mp = VarMu ? mu + ia : nullptr;
+  auto fetch = [&](int j) {
+    Row q = {};
+    const long long g = (long long)j * L.P;
+    if (in) {
+      q.u = *reinterpret_cast<const Two<T>*>(xp + L.off[0] + g);
+      q.v = *reinterpret_cast<const Two<T>*>(xp + L.off[1] + g);
+      if (VarMu) q.m = *reinterpret_cast<const Two<T>*>(mp + g);
+    }
+    return q;
+  };
+  // rows j - 1, j, j + 1 and the two after
+  const int jend = min(j0 + ky, L.n[1] - 1);
+  Row lo = {}, at = fetch(j0 - 1), up = fetch(j0), u2 = fetch(j0 + 1), u3 = {};
+  if (j0 + 2 <= jend) u3 = fetch(j0 + 2);
+  auto left = [](T w) { return __shfl_up_sync(0xffffffffu, w, 1); };
+  auto right = [](T w) { return __shfl_down_sync(0xffffffffu, w, 1); };
+  const bool own = lane >= 1 && lane <= 30;
+  const bool va = own && ia >= 1 && ia <= L.n[0] - 2, vb = own && ia + 1 >= 1 && ia + 1 <= L.n[0] - 2;
+  const T ws = Kc<T>::ws(L), g2 = Kc<T>::g2(L);
+  Two<T> dprev = {(T)0, (T)0};  // divergences of the row below
+  double dot = 0.0;
+#pragma unroll 1
+  for (int j = j0 - 1; j < jend; ++j) {
+    Row u4 = {};
+    if (j + 4 <= jend) u4 = fetch(j + 4);
+    // cells of row j, as neg_div_at forms them
+    Two<T> d = {(T)0, (T)0};
+    const T uR = right(at.u.a);
+    if (gd) {
+      d.a = at.u.a - at.u.b + at.v.a - up.v.a;
+      d.b = at.u.b - uR + at.v.b - up.v.b;
+    }
+    if (j >= j0) {
+      const T uL = left(at.u.b), vL = left(at.v.b), vR = right(at.v.a), dL = left(d.b);
+      Two<T> yu, yv;
+      if (!VarMu) {
+        auto row = [&](T xf, T e, T w, T n, T s, T dp, T dm) {
+          T acc = e + w + n + s;
+          return const_row<T, 1>(L, (T)0, xf, acc, gd, dp, dm);
+        };
+        yu.a = row(at.u.a, at.u.b, uL, up.u.a, lo.u.a, d.a, dL);
+        yu.b = row(at.u.b, uR, at.u.a, up.u.b, lo.u.b, d.b, d.a);
+        yv.a = row(at.v.a, at.v.b, vL, up.v.a, lo.v.a, d.a, dprev.a);
+        yv.b = row(at.v.b, vR, at.v.a, up.v.b, lo.v.b, d.b, dprev.b);
+      } else {
+        // cells: c this row, s the row below, n above; l / r the columns beside
+        const Two<T> c = at.m, s = lo.m, n = up.m;
+        const T cl = left(c.b), sl = left(s.b), nl = left(n.b), cr = right(c.a), sr = right(s.a);
+        // link by link in w_row_var_deep's order
+        auto row = [&](T xf, T m0, T x0, T m1, T x1, T mp, T xp, T mm, T xm, T dp, T dm) {
+          T acc = 0;
+          acc = fma(m0, xf - x0, acc);
+          acc = fma(m1, xf - x1, acc);
+          acc = fma(mp, xf - xp, acc);
+          acc = fma(mm, xf - xm, acc);
+          T w = mul_rn(acc, ws);
+          return gd ? fma(g2, dp - dm, w) : w;
+        };
+        auto mean = [](T p, T q, T o, T z) { return (((p + q) + o) + z) / (T)4; };
+        const T ka = mean(sl, cl, s.a, c.a), kb = mean(s.a, c.a, s.b, c.b);  // nodes (i, j): u's order
+        yu.a = row(at.u.a, c.a, at.u.b, cl, uL, mean(cl, nl, c.a, n.a), up.u.a, ka, lo.u.a, d.a, dL);
+        yu.b = row(at.u.b, c.b, uR, c.a, at.u.a, mean(c.a, n.a, c.b, n.b), up.u.b, kb, lo.u.b, d.b, d.a);
+        yv.a = row(at.v.a, c.a, up.v.a, s.a, lo.v.a, mean(s.a, s.b, c.a, c.b), at.v.b, mean(sl, s.a, cl, c.a), vL, d.a, dprev.a);
+        yv.b = row(at.v.b, c.b, up.v.b, s.b, lo.v.b, mean(s.b, sr, c.b, cr), vR, mean(s.a, s.b, c.a, c.b), at.v.a, d.b, dprev.b);
+      }
+      T* yp = y + (long long)j * L.P + ia;
+      const T w[8] = {at.u.a, yu.a, at.v.a, yv.a, at.u.b, yu.b, at.v.b, yv.b};
+      double z[8];
+      to_f64(w, z);
+      if (va) dot = fma(z[0], z[1], fma(z[2], z[3], dot));
+      if (vb) dot = fma(z[4], z[5], fma(z[6], z[7], dot));
+      if (va && vb) {
+        *reinterpret_cast<Two<T>*>(yp + L.off[0]) = yu;
+        *reinterpret_cast<Two<T>*>(yp + L.off[1]) = yv;
+      } else if (va) {
+        yp[L.off[0]] = yu.a;
+        yp[L.off[1]] = yv.a;
+      } else if (vb) {
+        yp[L.off[0] + 1] = yu.b;
+        yp[L.off[1] + 1] = yv.b;
+      }
+    }
+    dprev = d;
+    lo = at;
+    at = up;
+    up = u2;
+    u2 = u3;
+    u3 = u4;
+  }
+  return dot;
+}
+
+// position t of the shell: the rows 0, n - 1 and n whole, then the columns 0,
+// n - 1 and n of the others
+template <typename T, bool VarMu>
+__device__ __forceinline__ double mac2_shell_body(const Lvl& L, int wonly, const T* GKB_RESTRICT x, T* GKB_RESTRICT y,
+                                                  int t) {
+  const int w = L.n[0] + 1, h = L.n[1] - 2;
+  int i, j;
+  if (t < 3 * w) {
+    const int q = t / w;
+    i = t - q * w;
+    j = q == 0 ? 0 : L.n[1] - 2 + q;
+  } else {
+    t -= 3 * w;
+    if (t >= 3 * h) return 0.0;
+    const int q = t / h;
+    j = 1 + t - q * h;
+    i = q == 0 ? 0 : L.n[0] - 2 + q;
+  }
+  const bool gd = L.has_gd && !wonly;
+  const T g2 = Kc<T>::g2(L);
+  const int p[3] = {i, j, 0};
+  const long long cb = cix(L, i, j, 0);
+  const T d0 = gd ? neg_div<T>(L, x, i, j, 0) : (T)0;
+  double dot = 0.0;
+#define GKB_MAC2_SHELL(C, DMINUS)                                                                          \
+  if (in_store<C>(L, i, j, 0)) {                                                                           \
+    const long long id = L.off[C] + cb;                                                                    \
+    T val = 0;                                                                                             \
+    if (face_active<C>(L, i, j, 0)) {                                                                      \
+      const T xf = x[id];                                                                                  \
+      const T dm = gd ? (DMINUS) : (T)0;                                                                   \
+      if (VarMu) {                                                                                         \
+        val = mul_rn(w_row<T, VarMu, C>(L, x, p, xf), Kc<T>::ws(L));                                       \
+        if (gd) val = fma(g2, d0 - dm, val);                                                               \
+      } else if (const_regular<C>(L, p)) {                                                                 \
+        val = const_row<T, 1>(L, (T)0, xf, nb_sum<T>(L, x + id), gd, d0, dm);                              \
+      } else {                                                                                             \
+        val = wall_row<T>(w_row<T, false, C>(L, x, p, xf), Kc<T>::ws(L), gd, g2, d0, dm);                  \
+      }                                                                                                    \
+      dot = fma((double)xf, (double)val, dot);                                                             \
+    }                                                                                                      \
+    y[id] = val;                                                                                           \
+  }
+  GKB_MAC2_SHELL(0, neg_div<T>(L, x, i - 1, j, 0))
+  GKB_MAC2_SHELL(1, neg_div<T>(L, x, i, j - 1, 0))
+#undef GKB_MAC2_SHELL
+  return dot;
+}
+
+template <typename T, bool VarMu>
+__device__ __forceinline__ void mac2_body(const Blk& B, const Lvl& L, int wonly, const T* GKB_RESTRICT x,
+                                          T* GKB_RESTRICT y, RedBuf red, int fin, void* st) {
+  const int by = mac2_box_y(L);
+  double v[1];
+  if ((int)B.y < by) v[0] = mac2_box_body<T, VarMu>(B, L, wonly, x, y);
+  else v[0] = mac2_shell_body<T, VarMu>(L, wonly, x, y, (int)(((B.y - by) * B.nx + B.x) * (BX * BY) + threadIdx.y * BX + threadIdx.x));
+  grid_reduce<1>(v, red, fin, st, B);
+}
+
+template <typename T, bool VarMu>
+__global__ void __launch_bounds__(BX* BY, 2) k_mac2(const __grid_constant__ Lvl L, int wonly, const T* GKB_RESTRICT x,
+                                                    T* GKB_RESTRICT y, RedBuf red, int fin, void* st) {
+  mac2_body<T, VarMu>(native_blk(), L, wonly, x, y, red, fin, st);
 }
 
 // levels that take the split kernels (smaller ones stay with k_mac_tile)
@@ -638,7 +866,8 @@ __device__ __forceinline__ double mac3_shell_body(const Lvl& L, int wonly, const
 template <typename T, int MODE, bool DOT>
 __global__ void __launch_bounds__(BX* BY, sizeof(T) == 8 ? 3 : 4) k_mac3(Lvl L, int wonly, const T* GKB_RESTRICT x,
                                                     const T* GKB_RESTRICT b, T* GKB_RESTRICT y, RedBuf red,
-                                                    int fin, void* st) {
+                                                    int fin, void* st, const int* pred) {
+  if (pred && !*pred) return;  // predicated launch (uniform over the grid)
   const int bz = mac3_box_z(L);
   double dot;
   if ((int)blockIdx.z < bz) {

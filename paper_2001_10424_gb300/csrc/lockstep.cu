@@ -101,6 +101,15 @@ __global__ void __launch_bounds__(BX* BY) kb_tile(const JTile<T>* jobs, const un
   LS_RUN(JTile<T>, mac_tile_body<T, false, MODE, DOT>(B, job.L, job.wonly, job.x, job.b, job.y, job.red, job.fin, job.st, nullptr))
 }
 
+// y = M x and x . y, in the form that Ops::apply_dot takes for the level
+template <typename T>
+__global__ void __launch_bounds__(BX* BY, 2) kb_apply_dot(const JTile<T>* jobs, const unsigned* map) {
+  LS_RUN(JTile<T>, if (mac2_level<T>(job.L)) mac2_body<T, false>(B, job.L, job.wonly, job.x, job.y, job.red, job.fin, job.st);
+         else mac_tile_body<T, false, 1, true>(B, job.L, job.wonly, job.x, job.b, job.y, job.red, job.fin, job.st, nullptr))
+}
+template <typename T>
+inline dim3 apply_dot_grid(const Lvl& L) { return mac2_level<T>(L) ? mac2_grid<T>(L) : face_grid(L); }
+
 // use2: the level takes the class-stencil smoother (as Ops::cheb decides)
 template <typename T>
 struct JCheb { JobHead h; Lvl L; const T* r; T* x; T* d; T ca, cb; int x_zero, use2; const T* table; Fold2In<T> fs; };
@@ -874,8 +883,8 @@ void Lockstep::Impl::cg_body(cudaStream_t st, cudaStream_t sc) {
       j.red = s.red;
       j.fin = FIN_CG_PAP;
       j.st = s.cg_dev;
-      return face_grid(s.L32);
-    }, kb_tile<float, 1, true>);
+      return apply_dot_grid<float>(s.L32);
+    }, kb_apply_dot<float>);
     launch<JCgUpd<float>>(st, GKB_KC_BLAS, ps, dim3(RB), [&](int p, JCgUpd<float>& j) {
       Solver& s = *S[p];
       j.h.active = G + p;
@@ -905,8 +914,8 @@ void Lockstep::Impl::cg_body(cudaStream_t st, cudaStream_t sc) {
       j.red = s.red;
       j.fin = FIN_CG_PAP;
       j.st = s.cg_dev;
-      return face_grid(s.L64);
-    }, kb_tile<double, 1, true>);
+      return apply_dot_grid<double>(s.L64);
+    }, kb_apply_dot<double>);
     launch<JCgUpd<double>>(st, GKB_KC_BLAS, ps, dim3(RB), [&](int p, JCgUpd<double>& j) {
       Solver& s = *S[p];
       j.h.active = G + p;
@@ -1020,8 +1029,8 @@ void Lockstep::Impl::capture(cudaStream_t st, cudaStream_t sb, cudaStream_t sc) 
       j.red = s.red;
       j.fin = FIN_STORE;
       j.st = (double*)((char*)s.gkb_dev + offsetof(GkbState, red));
-      return face_grid(s.L64);
-    }, kb_tile<double, 1, true>);
+      return apply_dot_grid<double>(s.L64);
+    }, kb_apply_dot<double>);
   };
   auto vec64 = [&](cudaStream_t s_, const int* G, int op, std::function<const double*(Solver&)> x,
                    std::function<double*(Solver&)> y, bool cells, double a = 0, double b = 0) {
