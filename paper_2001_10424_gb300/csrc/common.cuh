@@ -79,27 +79,29 @@ struct Blk {
 };
 
 #ifdef __CUDACC__
-// eight values in double. A float's conversion runs on the FP64 unit (16
+// N values in double. A float's conversion runs on the FP64 unit (16
 // cycles a warp and SM), which sums of products of floats in double keep busy
 // already; the bits of normal numbers move over with integer instructions.
 // With a zero, subnormal, infinity or NaN among them all are converted.
-__device__ __forceinline__ void to_f64(const double (&v)[8], double (&o)[8]) {
+template <int N>
+__device__ __forceinline__ void to_f64(const double (&v)[N], double (&o)[N]) {
 #pragma unroll
-  for (int k = 0; k < 8; ++k) o[k] = v[k];
+  for (int k = 0; k < N; ++k) o[k] = v[k];
 }
-__device__ __forceinline__ void to_f64(const float (&v)[8], double (&o)[8]) {
+template <int N>
+__device__ __forceinline__ void to_f64(const float (&v)[N], double (&o)[N]) {
   unsigned top = 0;  // 2 |bits| - 2^24 wraps below the smallest normal number
 #pragma unroll
-  for (int k = 0; k < 8; ++k) top = max(top, 2u * __float_as_uint(v[k]) - 0x01000000u);
+  for (int k = 0; k < N; ++k) top = max(top, 2u * __float_as_uint(v[k]) - 0x01000000u);
   if (top < 0xfe000000u) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
+    for (int k = 0; k < N; ++k) {
       const unsigned b = __float_as_uint(v[k]);
       o[k] = __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
     }
   } else {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) o[k] = (double)v[k];
+    for (int k = 0; k < N; ++k) o[k] = (double)v[k];
   }
 }
 

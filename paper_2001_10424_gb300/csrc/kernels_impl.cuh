@@ -803,6 +803,7 @@ __device__ __forceinline__ double mac3_box_body(const Blk& B, const Lvl& L, int 
           dlow = d0;
         }
       }
+      T pr[6];  // the factors of the position's three products
 #define GKB_MAC3_FACE(C, DPLUS, DMINUS)                                                        \
       {                                                                                        \
         const T xf = Xt[sc][C][ty + 1][tx + 1];                                                \
@@ -810,12 +811,18 @@ __device__ __forceinline__ double mac3_box_body(const Blk& B, const Lvl& L, int 
                 Xt[sc][C][ty][tx + 1];                                                         \
         acc += Xt[su][C][ty + 1][tx + 1] + Xt[sd][C][ty + 1][tx + 1];                          \
         const T val = const_row<T, MODE>(L, bv[C], xf, acc, gd, DPLUS, DMINUS);                \
-        if (DOT) dot += (double)xf * (double)val;                                              \
+        if (DOT) { pr[2 * C] = xf; pr[2 * C + 1] = val; }                                      \
         y[L.off[C] + cb] = val;                                                                \
       }
       GKB_MAC3_FACE(0, d0, dl)
       GKB_MAC3_FACE(1, d0, db)
       GKB_MAC3_FACE(2, d0, dk)
+      if (DOT) {  // converted together (FP32: 160^3 97.8 -> 67.4 us with its sum, 64^3 23.8 -> 21.9 us)
+        double z[6];
+        to_f64(pr, z);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) dot = fma(z[2 * c], z[2 * c + 1], dot);
+      }
 #undef GKB_MAC3_FACE
     }
   }
