@@ -142,12 +142,15 @@ typedef struct {
                              profiling)                                        */
   int profile;            /* 1: time every kernel launch with CUDA events on
                              the stream and report per-class totals in
-                             gkb_stats (adds event overhead between kernels)  */
+                             gkb_stats (adds event overhead between kernels;
+                             2D V-cycles run as separate launches of the same
+                             steps instead of the fused legs)                  */
   int kernel_variant;     /* stencil kernels' deep-interior fast paths (same
                              values bit for bit as the general paths, except
                              the 3D constant-viscosity smoother's folded
                              stencil, which agrees to rounding):
-                             0: on in FP32, off in FP64 (measured fastest);
+                             0: on in FP32 and, for 2D constant viscosity, in
+                             FP64, off in FP64 otherwise (measured fastest);
                              1: off everywhere; 2: on everywhere               */
   int unet_side;          /* GKB_INNER_FCG_UNET: longer side (cells) of the
                              multigrid level where the network replaces the
