@@ -425,7 +425,8 @@ __host__ __device__ __forceinline__ int mac2_ky(const Lvl& L) {
   return w >= 8 * fill ? 8 : w >= 4 * fill ? 4 : w >= 2 * fill ? 2 : 1;
 }
 
-// constant viscosity, or cell viscosities with N = n I and the Laplacian form
+// constant viscosity, or cell viscosities with N = n I and the Laplacian form;
+// a narrower grid would leave most of a strip's 60 columns empty
 template <typename T>
 __host__ __device__ __forceinline__ bool mac2_level(const Lvl& L) {
   const bool plain = sizeof(T) == 4 ? !L.nw32 && !L.em32 : !L.nw64 && !L.em64;

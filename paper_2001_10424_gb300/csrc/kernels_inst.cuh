@@ -57,6 +57,8 @@ void Ops<KT>::residual(const Lvl& L, const KT* x, const KT* b, KT* r, cudaStream
   if (mac3_level(L) && !GKB_VARMU(L) && x) {
     k_mac3<KT, 0, false><<<mac3_grid(L), dim3(BX, BY), 0, s>>>(L, 0, x, b, r, red, 0, nullptr, pred);
   } else if (pred && x) {
+    // (3D constant viscosity stays with the plane-walking kernel, whose grid is
+    // small by itself: looping tiles took 160^3 mixed from 617 to 628 ms)
     const dim3 g = face_grid(L);
     const unsigned nb = (unsigned)std::min<long long>((long long)g.x * g.y * g.z, 152 * 8);
     if (GKB_VARMU(L)) k_residual_if<KT, true><<<nb, dim3(BX, BY), 0, s>>>(L, g, x, b, r, pred);
