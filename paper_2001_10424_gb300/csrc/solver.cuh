@@ -47,7 +47,12 @@ struct DevBuf {
       throw Error{GKB_ERR_OOM, "cudaMalloc of " + std::to_string(count * sizeof(T)) + " bytes failed"};
     }
     n = count;
+    // the fill runs on the legacy stream, and returns before it is done: waited
+    // for, as the caller's kernels may run on a stream that does not wait for
+    // that one (the weight gradient's partial sums are allocated right before
+    // the kernel that writes them)
     GKB_CUDA(cudaMemset(p, 0, count * sizeof(T)));
+    GKB_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
   }
   void release() {
     if (p) cudaFree(p);
