@@ -771,6 +771,20 @@ static dim3 row_grid(int items, int rows) { return dim3((items + UT - 1) / UT, s
 // host side
 // ---------------------------------------------------------------------------
 
+// shared memory of an FP32 forward convolution of cin channels
+template <int COT, int CG, int RG>
+static size_t fwd_smem(int cin) {
+  return ((size_t)(cin + 3) / 4 * 4 * ConvSmem<RG>::plane + 9ull * cin * COT * CG) * sizeof(float);
+}
+// The limit belongs to the kernel, not to a launch: it is set once, for the
+// widest layer that takes the instance. Set per launch, another thread's
+// narrower layer could lower it between this thread's call and its launch.
+template <int COT, int CG, int RG>
+static void allow_fwd(int cin) {
+  GKB_CUDA(cudaFuncSetAttribute(k_conv_fwd<COT, CG, RG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)fwd_smem<COT, CG, RG>(cin)));
+}
+
 void Unet::init(int cin, int k1, int k2, int cout, unsigned long long seed, cudaStream_t s) {
   c_in = cin; c1 = k1; c2 = k2; c_out = cout; stream = s;
   if (!(cin >= 1 && cin <= 16 && k1 == 16 && k2 == 32 && cout >= 1 && cout <= 3))
@@ -802,6 +816,12 @@ void Unet::init(int cin, int k1, int k2, int cout, unsigned long long seed, cuda
   GKB_CUDA(cudaFuncSetAttribute(k_conv_fwd_tc<32, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcSmem<32, 32>::bytes));
   GKB_CUDA(cudaFuncSetAttribute(k_conv_fwd_tc<48, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcSmem<48, 16>::bytes));
   GKB_CUDA(cudaFuncSetAttribute(k_conv_fwd_tc<64, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcSmem<64, 32>::bytes));
+  allow_fwd<16, 1, 4>(16);
+  allow_fwd<16, 2, 4>(16);
+  allow_fwd<8, 2, 4>(48);
+  allow_fwd<8, 2, 1>(48);
+  allow_fwd<8, 4, 2>(64);
+  allow_fwd<8, 4, 1>(64);
   GKB_CUDA(cudaFuncSetAttribute(k_wgrad<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
   GKB_CUDA(cudaFuncSetAttribute(k_wgrad<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
   bf16_stale = true;
@@ -834,10 +854,7 @@ static bool fills(dim3 g) { return (long long)g.x * g.y * g.z >= 152; }
 
 template <int COT, int CG, int RG>
 static void launch_fwd(const ConvArgs& A, cudaStream_t s) {
-  const size_t sm = ((size_t)(A.cin + 3) / 4 * 4 * ConvSmem<RG>::plane + 9ull * A.cin * COT * CG) * sizeof(float);
-  if (sm > 48 * 1024)
-    GKB_CUDA(cudaFuncSetAttribute(k_conv_fwd<COT, CG, RG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  k_conv_fwd<COT, CG, RG><<<conv_grid(A, RG), 32 * CG * RG, sm, s>>>(A);
+  k_conv_fwd<COT, CG, RG><<<conv_grid(A, RG), 32 * CG * RG, fwd_smem<COT, CG, RG>(A.cin), s>>>(A);
 }
 template <int COT, int CG, int RG>
 static void conv_fwd32(const ConvArgs& A, cudaStream_t s) {

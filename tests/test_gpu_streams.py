@@ -47,3 +47,39 @@ def test_solve_set_up_on_its_own_stream(lib, n, prec):
         finally:
             gk.gkb_destroy(h)
     assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
+
+
+def test_networks_of_two_threads(lib):
+    """FP32 passes of several networks at once, each from its own thread: a
+    launch's shared memory does not depend on another thread's layers."""
+    import threading
+
+    import torch
+    gk = lib
+    n, h, w = 1, 8, 8
+    x = torch.randn(n, h, w, 3, device="cuda")
+    torch.cuda.synchronize()
+    nets = [gk.gkb_unet_create(3, 16, 32, 2, 7, torch.cuda.Stream().cuda_stream) for _ in range(4)]
+    ys = [torch.zeros(n, h, w, 2, device="cuda") for _ in nets]
+    torch.cuda.synchronize()
+    errors = []
+
+    def work(k):
+        try:
+            for _ in range(400):
+                gk.gkb_unet_forward(nets[k], x, n, h, w, ys[k], 0)
+        except Exception as e:  # noqa: BLE001 - reported below
+            errors.append(e)
+
+    try:
+        threads = [threading.Thread(target=work, args=(k,)) for k in range(len(nets))]
+        for th in threads:
+            th.start()
+        for th in threads:
+            th.join()
+        assert not errors, errors
+        torch.cuda.synchronize()
+        assert bool(ys[0].any()) and all(torch.equal(ys[0], y) for y in ys)
+    finally:
+        for u in nets:
+            gk.gkb_unet_destroy(u)
