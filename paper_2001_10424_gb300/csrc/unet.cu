@@ -458,23 +458,32 @@ __global__ void __launch_bounds__(TCT) k_conv_fwd_tc(In2 in, const __nv_bfloat16
 // backward
 // ---------------------------------------------------------------------------
 
-// Weight gradient: partial[blk][t], t < 9 cin co: the sum over this block's
-// pixels of in[p + tap, ci] dpre[p, co]; t in [9 cin co, 9 cin co + co): of
-// dpre. A contraction over the pixels, bound by the FP32 pipe once a thread
+// Weight gradient: rows of partial sums over pixels p of in[p + tap, ci]
+// dpre[p, co] (partial) and of dpre (bpart), which k_reduce_wgrad adds up in
+// FP64. A contraction over the pixels, bound by the FP32 pipe once a thread
 // owns all nine taps of one input channel and COW outputs: along a pixel row
 // it keeps the 3 x 3 window of its channel in registers, so a pixel costs
 // three new inputs and COW gradients for 9 COW multiply-adds (the window and
-// the gradients of a warp are consecutive words or broadcasts). G thread groups
-// share a block's rows and are summed in group order. On 8 images of 512^2:
-// 48 -> 16 1.43 ms (20 TFLOP/s; staging the bilinear input costs as much as
-// the sums), 16 -> 16 0.45 ms, 64 -> 32 at half resolution 0.68 ms; the nine
-// layers together 4.1 ms, a thread per weight on 8-pixel patches took 44 ms.
+// the gradients of a warp are consecutive words or broadcasts). The thread
+// groups of a block share its rows of pixels.
+//
+// An FP32 sum ends after `chain` pixels (wgrad_shape): the thread adds it to
+// its row of partials and starts again. A row holds 9 x T x COW values at
+// (tap T + thread) COW + output, so that a warp's sums are consecutive there.
+// On 8 images of 512^2: 48 -> 16 1.48 ms (20 TFLOP/s; staging the bilinear
+// input costs as much as the sums), 16 -> 16 0.48 ms, 64 -> 32 at half
+// resolution 0.72 ms; the nine layers with their reductions 4.0 ms, a thread
+// per weight on 8-pixel patches took 44 ms.
 constexpr int WGC = 32;  // columns of a tile
 struct WgradArgs {
   In2 in;
   const float* dpre;
   float* partial;
+  double* bpart;
   int cin, co, groups, ty, tiles, per_block, n, h, wd;  // ty: rows of a tile
+  int chain, per_row;        // pixels of an FP32 sum, sums added into a row of partials
+  int rows;                  // rows of partials of a thread group
+  int bgroups;               // rows of bpart of a block
 };
 
 template <int COW>
@@ -491,7 +500,36 @@ __global__ void __launch_bounds__(256, 2) k_wgrad(const WgradArgs A) {
   for (int q = 0; q < 9; ++q)
 #pragma unroll
     for (int o = 0; o < COW; ++o) acc[q][o] = 0.f;
-  float bsum = 0.f;  // thread t < co: sum of dpre over the block's pixels
+  double bsum = 0.0;  // thread t < co * bgroups: sum of dpre[., t % co]
+  const int nw = 9 * cin * co;
+  float* const rows = A.partial + ((long long)(blockIdx.x * A.groups + g) * A.rows) * nw + (long long)r * COW;
+  int done = 0, sums = 0;  // pixels of the current sum, sums written
+  auto flush = [&]() {
+    float* out = rows + (long long)(sums / A.per_row) * nw;
+    const bool first = sums % A.per_row == 0;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+      float* d = out + q * T * COW;
+      if constexpr (COW % 4 == 0) {
+#pragma unroll
+        for (int o = 0; o < COW; o += 4) {
+          float4 v = make_float4(acc[q][o], acc[q][o + 1], acc[q][o + 2], acc[q][o + 3]);
+          if (!first) {
+            const float4 u = *reinterpret_cast<const float4*>(d + o);
+            v = make_float4(u.x + v.x, u.y + v.y, u.z + v.z, u.w + v.w);
+          }
+          *reinterpret_cast<float4*>(d + o) = v;
+        }
+      } else {
+#pragma unroll
+        for (int o = 0; o < COW; ++o) d[o] = first ? acc[q][o] : d[o] + acc[q][o];
+      }
+#pragma unroll
+      for (int o = 0; o < COW; ++o) acc[q][o] = 0.f;
+    }
+    done = 0;
+    ++sums;
+  };
   const int tx = (A.wd + WGC - 1) / WGC, tyn = (A.h + A.ty - 1) / A.ty;
   const int t1 = min(A.tiles, (int)(blockIdx.x + 1) * A.per_block);
   for (int tile = blockIdx.x * A.per_block; tile < t1; ++tile) {
@@ -545,80 +583,115 @@ __global__ void __launch_bounds__(256, 2) k_wgrad(const WgradArgs A) {
           w[ky][0] = xp[ky * xrow];
           w[ky][1] = xp[ky * xrow + cin];
         }
+        const int seg = min(A.chain, WGC);
+        for (int xs0 = 0; xs0 < WGC; xs0 += seg) {
 #pragma unroll 4
-        for (int x = 0; x < WGC; ++x) {
+          for (int x = xs0; x < xs0 + seg; ++x) {
 #pragma unroll
-          for (int ky = 0; ky < 3; ++ky) w[ky][2] = xp[ky * xrow + (x + 2) * cin];
-          float d[COW];
-          if constexpr (COW % 4 == 0) {
+            for (int ky = 0; ky < 3; ++ky) w[ky][2] = xp[ky * xrow + (x + 2) * cin];
+            float d[COW];
+            if constexpr (COW % 4 == 0) {
 #pragma unroll
-            for (int o = 0; o < COW; o += 4) {
-              const float4 v = *reinterpret_cast<const float4*>(dp + x * co + o);
-              d[o] = v.x;
-              d[o + 1] = v.y;
-              d[o + 2] = v.z;
-              d[o + 3] = v.w;
+              for (int o = 0; o < COW; o += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(dp + x * co + o);
+                d[o] = v.x;
+                d[o + 1] = v.y;
+                d[o + 2] = v.z;
+                d[o + 3] = v.w;
+              }
+            } else {
+#pragma unroll
+              for (int o = 0; o < COW; ++o) d[o] = dp[x * co + o];
             }
-          } else {
 #pragma unroll
-            for (int o = 0; o < COW; ++o) d[o] = dp[x * co + o];
+            for (int q9 = 0; q9 < 9; ++q9)
+#pragma unroll
+              for (int o = 0; o < COW; ++o) acc[q9][o] = fmaf(w[q9 / 3][q9 % 3], d[o], acc[q9][o]);
+#pragma unroll
+            for (int ky = 0; ky < 3; ++ky) {
+              w[ky][0] = w[ky][1];
+              w[ky][1] = w[ky][2];
+            }
           }
-#pragma unroll
-          for (int q9 = 0; q9 < 9; ++q9)
-#pragma unroll
-            for (int o = 0; o < COW; ++o) acc[q9][o] = fmaf(w[q9 / 3][q9 % 3], d[o], acc[q9][o]);
-#pragma unroll
-          for (int ky = 0; ky < 3; ++ky) {
-            w[ky][0] = w[ky][1];
-            w[ky][1] = w[ky][2];
-          }
+          done += seg;
+          if (done == A.chain) flush();
         }
       }
     }
-    if (tid < co) {
-      float s = 0.f;
-      for (int px = 0; px < A.ty * WGC; ++px) s += ds[px * co + tid];
-      bsum += s;
+    // dpre alone: runs of at most `chain` pixels
+    if (tid < co * A.bgroups) {
+      const int tile_px = A.ty * WGC, run = min(A.chain, tile_px);
+      for (int p0 = tid / co * run; p0 < tile_px; p0 += A.bgroups * run) {
+        float b = 0.f;
+#pragma unroll 8
+        for (int px = p0; px < min(p0 + run, tile_px); ++px) b += ds[px * co + tid % co];
+        bsum += b;
+      }
     }
   }
-  // the groups' sums in group order, then this block's row of partials
-  const int nw = 9 * cin * co;
-  float* out = A.partial + (long long)blockIdx.x * (nw + co);
-  __syncthreads();
-  float* red = wg_sm;  // the first `nw` words of the tile storage (one group: straight to memory)
-  for (int k = 0; k < A.groups; ++k) {
-    if (g == k) {
-#pragma unroll
-      for (int q = 0; q < 9; ++q)
-#pragma unroll
-        for (int o = 0; o < COW; ++o) {
-          const int t = (q * cin + ci) * co + ob + o;
-          if (A.groups == 1) out[t] = acc[q][o];
-          else red[t] = k ? red[t] + acc[q][o] : acc[q][o];
-        }
-    }
-    __syncthreads();
+  if (mine) {
+    if (done) flush();
+    while (sums < A.rows * A.per_row) flush();  // zeros where the last block has fewer tiles
   }
-  if (A.groups > 1)
-    for (int t = tid; t < nw; t += NT) out[t] = red[t];
-  if (tid < co) out[nw + tid] = bsum;
+  if (tid < co * A.bgroups) A.bpart[(long long)blockIdx.x * co * A.bgroups + tid] = bsum;
 }
 
-// out[t] = sum over blocks of partial[blk][t] in FP64, in a fixed order: 8
-// row groups of a block (rows k, k + 8, ...), then the groups in order
-__global__ void __launch_bounds__(256) k_reduce_rows(const float* __restrict__ partial, int nblk, int ntot,
-                                                     float* __restrict__ out) {
-  __shared__ double sh[8][32];
-  const int c = threadIdx.x & 31, k = threadIdx.x >> 5, t = blockIdx.x * 32 + c;
+// The rows of partials added in a fixed order: WG_RG row groups of a block
+// (rows k, k + WG_RG, ...), then the groups in FP64. Blocks [0, wblocks): the
+// weights' sums, from the order of a row (T threads of cow outputs) to
+// [tap][ci][co]; the others: the biases'.
+//
+// Within a group a sum is a pair of floats: Knuth's two-sum gives a value and
+// the exact error of every addition, the errors are added up beside it. That
+// keeps 2^-47 of the largest partial sum and runs on the FP32 pipe; in FP64
+// a thousand rows held that unit for 40 to 100 us a layer (1 x 512^2: 1.12 ms
+// for the nine layers' weight gradients, now 0.81). Sums that leave FP32's
+// range are formed in FP64.
+constexpr int WG_RC = 8, WG_RG = 32;  // columns and row groups of a block
+struct ReduceArgs {
+  const float* partial;
+  const double* bpart;
+  float* out;
+  int nrows, brows, cin, co, cow, wblocks;
+};
+__global__ void __launch_bounds__(WG_RC* WG_RG) k_reduce_wgrad(const ReduceArgs A) {
+  __shared__ double sh[WG_RC * WG_RG / 32][WG_RC];
+  const int c = threadIdx.x % WG_RC, k = threadIdx.x / WG_RC;
+  const bool bias = (int)blockIdx.x >= A.wblocks;
+  const int t = ((int)blockIdx.x - (bias ? A.wblocks : 0)) * WG_RC + c;
+  const int nw = 9 * A.cin * A.co, nt = bias ? A.co : nw;
   double s = 0.0;
-  if (t < ntot)
+  if (t < nt) {
+    if (bias) {
+#pragma unroll 8
+      for (int b = k; b < A.brows; b += WG_RG) s += A.bpart[(long long)b * A.co + t];
+    } else {
+      float hi = 0.f, lo = 0.f;
 #pragma unroll 16
-    for (int b = k; b < nblk; b += 8) s += partial[(long long)b * ntot + t];
-  sh[k][c] = s;
+      for (int b = k; b < A.nrows; b += WG_RG) {
+        const float v = A.partial[(long long)b * nw + t];
+        const float z = hi + v, w = z - hi;
+        lo += (hi - (z - w)) + (v - w);
+        hi = z;
+      }
+      s = (double)hi + (double)lo;
+      if (!isfinite(s)) {
+        s = 0.0;
+        for (int b = k; b < A.nrows; b += WG_RG) s += A.partial[(long long)b * nw + t];
+      }
+    }
+  }
+  for (int o = 16; o >= WG_RC; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) < WG_RC) sh[threadIdx.x >> 5][c] = s;
   __syncthreads();
-  if (k == 0 && t < ntot) {
-    for (int q = 1; q < 8; ++q) s += sh[q][c];
-    out[t] = (float)s;
+  if (k == 0 && t < nt) {
+    for (int q = 1; q < WG_RC * WG_RG / 32; ++q) s += sh[q][c];
+    int at = nw + t;
+    if (!bias) {
+      const int T = A.cin * (A.co / A.cow), o = t % A.cow, r = t / A.cow % T, tap = t / (A.cow * T);
+      at = (tap * A.cin + r % A.cin) * A.co + r / A.cin * A.cow + o;
+    }
+    A.out[at] = (float)s;
   }
 }
 
@@ -921,10 +994,18 @@ const float* Unet::forward(UnetAct& A, const float* x, int n, int h, int w, bool
   return A.y.p;
 }
 
-// Launch shape of layer L's weight gradient on n images of h x w. A thread's
-// sum runs over at most 512 pixels before it leaves for the FP64 sum over the
-// blocks (longer chains round worse than the 8-pixel partial sums they
-// replace), as long as that takes no more than WG_ROWS blocks.
+// Launch shape of layer L's weight gradient on n images of h x w, N pixels.
+//
+// Rounding: an FP32 sum of F terms leaves an error of about sqrt(F / 2) units
+// of its last place, and the sums of R / F of them in a row sqrt(R / (2 F)).
+// The bound kept is that of sums over 8 pixels added up by 304 blocks,
+// 8 + N / 2432 for F: F is the largest power of two below 3/4 of it, which
+// leaves room for the additions into a row, at least 8. A row takes
+// R = N / 1024 pixels per thread group (a power of two, at least F; up to four
+// groups count), so that about 1024 rows of a group are written and added up.
+// Against one sum per thread over all its pixels (128 to 2048), which was up
+// to five times as far off as the 8-pixel sums, a training step of 1 x 128^2
+// takes 0.82 ms in place of 0.76, one of 8 x 512^2 9.74 in place of 9.95.
 constexpr int WG_ROWS = 1024;
 // Outputs per thread: 4 (registers for 24 warps per SM), 8 where 4 would need
 // more threads than a block has, 2 where so few channels leave threads idle.
@@ -944,26 +1025,36 @@ static WgradArgs wgrad_shape(const ConvLayer& L, int n, int h, int w) {
   A.groups = std::max(1, std::min(8, 256 / T));
   A.ty = std::max(4, A.groups);
   A.tiles = n * ((w + WGC - 1) / WGC) * ((h + A.ty - 1) / A.ty);
+  const long long N = (long long)n * h * w;
+  A.chain = 8;
+  while (2 * A.chain <= 6 + 3 * N / 9728) A.chain *= 2;
+  long long row = A.chain;  // pixels of a row of partials
+  while (row * WG_ROWS * std::min(A.groups, 4) < N) row *= 2;
+  A.per_row = (int)(row / A.chain);
   const int px = WGC * A.ty / A.groups;  // pixels of a tile per thread
-  A.per_block = std::max(1, std::min(512 / px, A.tiles / 608));
-  A.per_block = std::max(A.per_block, (A.tiles + WG_ROWS - 1) / WG_ROWS);
+  A.per_block = (int)std::max(1LL, row / px);
+  A.rows = (int)std::max(1LL, px / row);
+  const int runs = (WGC * A.ty + A.chain - 1) / A.chain;  // runs of dpre sums in a tile
+  A.bgroups = std::min(runs, std::max(1, T * A.groups / L.cout));
   return A;
 }
 
 // weight gradient of layer li into grads (two deterministic passes)
 static void conv_bwd_w(Unet& U, int li, In2 in, const float* dpre, int n, int h, int w) {
   const ConvLayer& L = U.layers[li];
-  const int ntot = (int)(L.nw() + L.cout);
   WgradArgs A = wgrad_shape(L, n, h, w);
   A.in = in;
   A.dpre = dpre;
   const int nblk = (A.tiles + A.per_block - 1) / A.per_block;
-  if (U.wpart.n < (size_t)nblk * ntot) U.wpart.alloc((size_t)nblk * ntot);
+  const size_t np = (size_t)nblk * A.groups * A.rows * L.nw(), nb = (size_t)nblk * A.bgroups * L.cout;
+  if (U.wpart.n < np) U.wpart.alloc(np);
+  if (U.bpart.n < nb) U.bpart.alloc(nb);
   A.partial = U.wpart.p;
+  A.bpart = U.bpart.p;
   const int cow = wgrad_cow(L), T = L.cin * (L.cout / cow);
   const int nt = (std::max(T * A.groups, L.cout) + 31) / 32 * 32;
   const size_t tile = ((size_t)(A.ty + 2) * (WGC + 2) * L.cin + 3) / 4 * 4 + (size_t)A.ty * WGC * L.cout;
-  const size_t sm = std::max(tile, A.groups > 1 ? (size_t)L.nw() : (size_t)0) * sizeof(float);
+  const size_t sm = tile * sizeof(float);
   cudaStream_t s = U.stream;
   ProfScope ps_(GKB_KC_UNET, s, (long long)n * h * w);
   if (cow == 8) k_wgrad<8><<<nblk, nt, sm, s>>>(A);
@@ -971,7 +1062,9 @@ static void conv_bwd_w(Unet& U, int li, In2 in, const float* dpre, int n, int h,
   else if (cow == 3) k_wgrad<3><<<nblk, nt, sm, s>>>(A);
   else if (cow == 2) k_wgrad<2><<<nblk, nt, sm, s>>>(A);
   else k_wgrad<1><<<nblk, nt, sm, s>>>(A);
-  k_reduce_rows<<<(ntot + 31) / 32, 256, 0, s>>>(U.wpart.p, nblk, ntot, U.grads.p + L.off);
+  const int wb = (int)((L.nw() + WG_RC - 1) / WG_RC);
+  const ReduceArgs R{U.wpart.p, U.bpart.p, U.grads.p + L.off, nblk * A.groups * A.rows, nblk * A.bgroups, L.cin, L.cout, cow, wb};
+  k_reduce_wgrad<<<wb + (L.cout + WG_RC - 1) / WG_RC, WG_RC * WG_RG, 0, s>>>(R);
   GKB_CUDA(cudaGetLastError());
 }
 

@@ -41,7 +41,8 @@ struct Unet {
   // backward scratch
   int gn = 0, gh = 0, gw = 0;
   DevBuf<float> g_full0, g_full1, g_half0, g_half1, g_q0, g_q1, g_e;
-  DevBuf<float> wpart;                  // per-block partial weight gradients
+  DevBuf<float> wpart;                  // partial sums of the weight gradients
+  DevBuf<double> bpart;                 // and of the bias gradients
   DevBuf<double> red_partial;
   DevBuf<unsigned int> red_ticket;
   DevBuf<double> loss_dev;
