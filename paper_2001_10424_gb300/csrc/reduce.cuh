@@ -63,12 +63,10 @@ __device__ void grid_reduce(double (&v)[NV], RedBuf red, int fin, void* st, cons
   const unsigned bid = B.x + B.nx * (B.y + B.ny * B.z);
   const unsigned nblk = B.nx * B.ny * B.nz;
   double s = block_sum<NV>(v, sh, tid, nthr);
-  if (warp < NV && lane == 0) {
-    red.partial[(size_t)bid * NV + warp] = s;
-    __threadfence();
-  }
+  if (warp < NV && lane == 0) red.partial[(size_t)bid * NV + warp] = s;
   __syncthreads();
   if (tid == 0) {
+    __threadfence();  // the block's partials, ordered before its ticket
     unsigned t = atomicAdd(red.ticket, 1u);
     am_last = (t == nblk - 1);
   }
