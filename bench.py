@@ -492,6 +492,20 @@ def roofline(gk, torch, wk, args, form, hbm_peak, peak_kind):
     torch.cuda.synchronize()
     torch.cuda.profiler.stop()
     B.destroy()
+    how = "%d problem(s), profiled host-sequenced solve" % n_profiled
+    run_ms = None
+    if wk.dim == 2:
+        # the classes above are those of a V-cycle's separate steps, which have
+        # algorithmic bytes and flops of their own; a 2D solve fuses a level's
+        # steps into legs: the time per class of the launches that it makes
+        how += ", every step of a V-cycle its own launch"
+        B = Bound(gk, torch, wk, form, profile=2, subset=subset, autotune=args.autotune)
+        run_ms = {}
+        for i, h in enumerate(B.hs):
+            gk.gkb_solve(h, B.g[i], B.r[i], args.tol, args.delay, B.w[i], B.p[i], B.w0[i], B.p0[i])
+            for k, v in gk.gkb_stats(h)["kernel_ms"].items():
+                run_ms[k] = round(run_ms.get(k, 0.0) + v, 3)
+        B.destroy()
     table = PER_UNIT[wk.dim]
     cand = {k: v for k, v in ms.items() if k in table or (k == "unet" and wk.learned)}
     top = max(cand, key=cand.get)
@@ -511,7 +525,9 @@ def roofline(gk, torch, wk, args, form, hbm_peak, peak_kind):
         rl["share_of_kernel_time"] = ms[top] / total_ms if total_ms else None
         rl["traffic"] = TRAFFIC.get((wk.name, form, top))
         rl["class_ms"] = {k: round(v, 3) for k, v in ms.items()}
-        rl["profiled"] = "%d problem(s), profiled host-sequenced solve" % n_profiled
+        if run_ms:
+            rl["class_ms_fused_legs"] = run_ms
+        rl["profiled"] = how
         return rl
     varmu = any(not np.isscalar(p["mu"]) for p in wk.problems)
     per_unit_bytes = table[top][1] + (VARMU_SMOOTH_EXTRA[wk.dim] if (top == "smooth" and varmu) else 0.0)
@@ -536,7 +552,9 @@ def roofline(gk, torch, wk, args, form, hbm_peak, peak_kind):
         rl["traffic_basis"] = "ncu DRAM read+write of one finest-level launch (cold cache)"
         rl["traffic_algorithmic"] = m0 * (CAPTURED_ELEMS.get(top, table[top][1]) + extra) * s
     rl["class_ms"] = {k: round(v, 3) for k, v in ms.items()}
-    rl["profiled"] = "%d problem(s), profiled host-sequenced solve" % n_profiled
+    if run_ms:
+        rl["class_ms_fused_legs"] = run_ms
+    rl["profiled"] = how
     rl["flops_per_unit"] = flops / max(1, units[top])
     # the same class restricted to its finest-level launches (the level the
     # ncu captures look at; the class figure above averages every level,

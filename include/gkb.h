@@ -142,9 +142,12 @@ typedef struct {
                              profiling)                                        */
   int profile;            /* 1: time every kernel launch with CUDA events on
                              the stream and report per-class totals in
-                             gkb_stats (adds event overhead between kernels;
-                             2D V-cycles run as separate launches of the same
-                             steps instead of the fused legs)                  */
+                             gkb_stats (adds event overhead between kernels),
+                             2D V-cycles as separate launches of their steps,
+                             so that every step shows in its own class;
+                             2: the same, with the launches that a solve
+                             without profiling makes: a fused leg counts under
+                             GKB_KC_SMOOTH, its work the level's unknowns      */
   int kernel_variant;     /* stencil kernels' deep-interior fast paths (same
                              values bit for bit as the general paths, except
                              the 3D constant-viscosity smoother's folded

@@ -1687,7 +1687,7 @@ void Solver::build_inner() {
   gmg32.cheb_lo = gmg64.cheb_lo = opt.cheb_lo;
   gmg32.cheb_hi = gmg64.cheb_hi = opt.cheb_hi;
   gmg32.tail_side = gmg64.tail_side = opt.tail_side;
-  gmg32.legs = gmg64.legs = !opt.profile;
+  gmg32.legs = gmg64.legs = opt.profile != 1;
   if (mixed) {
     if (use_gmg) gmg32.build(L32, mu32.p, opt.coarse_max, opt.smoother_degree, red, scal.p, stream);
     cg32.init(L32, use_gmg ? &gmg32 : nullptr, red, cg_dev, cg_host);

@@ -111,7 +111,7 @@ struct Gmg {
   // viscosity): levels from tail_level on (the first whose longer side is at
   // most tail_side) run inside k_vtail; -1: off
   int tail_side = 0;
-  bool legs = true;   // fused legs where a level qualifies (off while profiling: every step its own launch)
+  bool legs = true;   // fused legs where a level qualifies (off with profile = 1: every step its own launch)
   int tail_level = -1;
   int tail_cs = 0;
   DevBuf<unsigned char> tail_buf;
