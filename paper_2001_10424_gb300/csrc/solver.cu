@@ -1687,7 +1687,7 @@ void Solver::build_inner() {
   gmg32.cheb_lo = gmg64.cheb_lo = opt.cheb_lo;
   gmg32.cheb_hi = gmg64.cheb_hi = opt.cheb_hi;
   gmg32.tail_side = gmg64.tail_side = opt.tail_side;
-  gmg32.legs = gmg64.legs = opt.profile != 1;
+  gmg32.legs = gmg64.legs = tuning || opt.profile != 1;
   if (mixed) {
     if (use_gmg) gmg32.build(L32, mu32.p, opt.coarse_max, opt.smoother_degree, red, scal.p, stream);
     cg32.init(L32, use_gmg ? &gmg32 : nullptr, red, cg_dev, cg_host);
@@ -1796,7 +1796,9 @@ void tune_read_file() {
 // (0.05 .. 0.3 of lambda_max) one after another, each by the device
 // time of a whole inner solve to tol_inner, and keep the fastest; results are
 // cached per device, grid, viscosity kind, precision, inner solver and gamma
-// decade, in the process and (GKB_TUNE_CACHE) in a text file.
+// decade, in the process and (GKB_TUNE_CACHE) in a text file. A profiled
+// handle's candidates make the launches of a solve without profiling too:
+// handles of either kind share the cached choice.
 void Solver::autotune_inner(bool var_mu, int weighted) {
   int dev = 0;
   GKB_CUDA(cudaGetDevice(&dev));
@@ -1837,6 +1839,11 @@ void Solver::autotune_inner(bool var_mu, int weighted) {
     opt.tail_side = tail;
     double ms = 1e300;
     int its = 0;
+    struct Building {
+      bool& on;
+      ~Building() { on = false; }
+    } building{tuning};
+    tuning = true;
     try {
       build_inner();
       ms = time_inner_solve(&its);

@@ -268,6 +268,7 @@ struct Solver {
   bool learned_inner() const { return opt.inner == GKB_INNER_FCG_UNET || opt.inner == GKB_INNER_FCG_UNET_MG; }
   void set_net(Unet* u);
   double tuned_ms = 0;            // inner-solve time of the tuned configuration
+  bool tuning = false;            // a candidate of the autotuner is being built and timed
   bool fast64() const;
   void build_inner();
   double time_inner_solve(int* its = nullptr);  // device ms of one inner solve (best of 3)

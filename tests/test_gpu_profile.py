@@ -31,3 +31,27 @@ def test_profile_of_the_launches_of_a_solve(lib, n, prec, var):
         assert (timed["kernel_ms"][k] > 0) == (count > 0), k
     fused = len(n) == 2
     assert (sum(steps["kernel_launches"].values()) > sum(ran["kernel_launches"].values())) == fused
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_profiled_handles_tune_the_same_launches(lib, prec):
+    """A profiled handle's choice is the cached one of every other handle of its
+    key, so it is made with the launches of a solve without profiling. A grid
+    and its transposed (another key, the same work) are timed within 40 % of
+    each other; with separate launches the profiled one took twice as long."""
+    import torch
+    gk = lib
+    ms = []
+    for n, profile in (((112, 80), 1), ((80, 112), 0)):
+        opt = gk.gkb_default_options()
+        opt.precision = prec
+        opt.autotune = 1
+        opt.profile = profile
+        opt.stream = torch.cuda.current_stream().cuda_stream
+        h = gk.gkb_create(opt)
+        try:
+            gk.gkb_set_problem(h, gk.make_grid(n, 1.0 / n[0], (0,) * 4), None, 1.0, 30.0, 0.0)
+            ms.append(gk.gkb_stats(h)["tuned_inner_ms"])
+        finally:
+            gk.gkb_destroy(h)
+    assert 1 / 1.4 <= ms[0] / ms[1] <= 1.4, ms
