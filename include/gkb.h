@@ -154,7 +154,11 @@ typedef struct {
                              stencil, which agrees to rounding):
                              0: on in FP32 and, for 2D constant viscosity, in
                              FP64, off in FP64 otherwise (measured fastest);
-                             1: off everywhere; 2: on everywhere               */
+                             1: off everywhere; 2: on everywhere (in FP64
+                             2D constant viscosity's products take theirs from
+                             2^19 cells up). With 1, small unpreconditioned CG
+                             solves also run on the general cluster kernel
+                             (same bits)                                       */
   int unet_side;          /* GKB_INNER_FCG_UNET: longer side (cells) of the
                              multigrid level where the network replaces the
                              rest of the V-cycle; 0: the finest level (the

@@ -1983,7 +1983,11 @@ void Solver::launch_cg_block(const double* fpad, double* xpad, cudaStream_t s) {
   const double tol2 = opt.tol_inner * opt.tol_inner;
   const bool var = L64.mu64 != nullptr;
   // every vector on chip where a block's copy of r and the threads' entries
-  // have room
+  // have room (us per iteration, k_cg_cluster -> on chip: 2D constant viscosity
+  // 32^2 9.3 -> 5.2, 62 x 60 11.2 -> 6.8; variable 16^2 10.2 -> 4.7, 62 x 60
+  // 12.0 -> 7.2; 3D constant 4^3 12.3 -> 6.2, 10^3 13.6 -> 7.0, 31 x 7 x 5
+  // 11.4 -> 8.1; variable 4^3 14.7 -> 6.2, 10^3 16.1 -> 7.2, 31 x 7 x 5 13.5 ->
+  // 8.4); kernel_variant 1 keeps the general kernel, which has the same bits
   constexpr size_t max_sm = 190 * 1024;
   const bool d3 = L64.dim == 3;
   auto sm_fn = d3 ? (var ? k_cg_cluster_sm<3, true> : k_cg_cluster_sm<3, false>)
@@ -1993,7 +1997,7 @@ void Solver::launch_cg_block(const double* fpad, double* xpad, cudaStream_t s) {
   const long long vch = (L64.nvel + cs - 1) / cs, pch = (npos + cs - 1) / cs, dim = L64.dim;
   const size_t sm = (size_t)(L64.nvel + 1 + vch + dim * pch) * sizeof(double) + (size_t)(dim * pch) * sizeof(int);
   const bool chip = L64.nvel <= CGS_LEN && vch <= CGS_E * SB && pch <= CGS_Q * SB && dim * pch <= CGS_F * SB &&
-                    sm <= max_sm && !L64.sym;
+                    sm <= max_sm && !L64.sym && opt.kernel_variant != 1;
   const void* fn = var ? (const void*)k_cg_cluster<true> : (const void*)k_cg_cluster<false>;
   if (!chip) cs = cg_cluster_size(fn, var ? 1 : 0, 0, SB);
   cudaLaunchConfig_t cfg = {};
