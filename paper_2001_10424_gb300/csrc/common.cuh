@@ -105,6 +105,29 @@ __device__ __forceinline__ void to_f64(const float (&v)[N], double (&o)[N]) {
   }
 }
 
+// 1 / b as its rounded value and the rest of it (the remainder 1 - b y of a
+// correctly rounded y is exact)
+struct Recip {
+  double y, lo;
+};
+__device__ __forceinline__ Recip recip(double b) {
+  const double y = 1.0 / b;
+  return {y, y * fma(-b, y, 1.0)};
+}
+// a / b, rounded as the division rounds, from r = recip(b) (Markstein: with
+// y = 1 / b rounded to nearest and a q less than an ulp off a / b, the remainder
+// a - b q is exact and q plus its quotient by y rounds correctly). a y alone
+// can be 1.5 ulps off; with the rest of 1 / b q is within 0.5 and a little.
+// Outside the exponents where no term under- or overflows: the division itself.
+__device__ __forceinline__ double div_by(double a, double b, Recip r) {
+  // biased exponents within 500 of 1 (integer tests: a comparison on the FP64
+  // unit costs as much as a multiply-add)
+  const unsigned ea = ((unsigned)__double2hiint(a) >> 20) & 0x7ff, eb = ((unsigned)__double2hiint(b) >> 20) & 0x7ff;
+  if (ea - 523u > 1000u || eb - 523u > 1000u) return a / b;
+  const double q = fma(a, r.y, a * r.lo);
+  return fma(fma(-b, q, a), r.y, q);
+}
+
 __device__ __forceinline__ Blk native_blk() {
   return Blk{blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x, gridDim.y, gridDim.z};
 }
