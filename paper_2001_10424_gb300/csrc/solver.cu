@@ -2537,7 +2537,10 @@ void Solver::apply(int op, const double* xin, double* yout) {
   double* dst = ydev ? yout : (out_cells ? stage_n.p : stage_m.p);
   if (op < GKB_OP_W || op > GKB_OP_M) throw Error{GKB_ERR_INVALID_ARG, "unknown operator"};
   // constant viscosity: straight between the compact vectors, unless the
-  // result would overwrite entries that other blocks still read
+  // result would overwrite entries that other blocks still read: a caller's
+  // vectors that overlap, and W and M between host vectors, whose input and
+  // output share stage_m. Those go through the padded arrays and the solver's
+  // own kernels
   if (!mu64.p && !overlap(src, nin, dst, nout)) {
     apply_compact(L, op, src, dst, s);
     if (!ydev) GKB_CUDA(cudaMemcpyAsync(yout, dst, nout * sizeof(double), cudaMemcpyDeviceToHost, s));
