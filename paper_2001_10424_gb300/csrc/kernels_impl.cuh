@@ -425,11 +425,13 @@ __host__ __device__ __forceinline__ int mac2_ky(const Lvl& L) {
   return w >= 8 * fill ? 8 : w >= 4 * fill ? 4 : w >= 2 * fill ? 2 : 1;
 }
 
-// constant viscosity, or cell viscosities with N = n I and the Laplacian form;
-// a narrower grid would leave most of a strip's 60 columns empty
+// constant viscosity or, in FP32, cell viscosities with N = n I and the
+// Laplacian form (FP64 levels with cell viscosities have a node table and keep
+// the tile kernel); a narrower grid would leave most of a strip's 60 columns
+// empty
 template <typename T>
 __host__ __device__ __forceinline__ bool mac2_level(const Lvl& L) {
-  const bool plain = sizeof(T) == 4 ? !L.nw32 && !L.em32 : !L.nw64 && !L.em64;
+  const bool plain = sizeof(T) == 4 ? !L.nw32 && !L.em32 : !L.mu64;
   return L.dim == 2 && L.fast && L.n[0] * (long long)L.n[1] >= Mac2<T>::MIN && L.n[0] >= 48 && L.n[1] >= 8 && !L.sym && plain;
 }
 __host__ __device__ __forceinline__ int mac2_box_y(const Lvl& L) {

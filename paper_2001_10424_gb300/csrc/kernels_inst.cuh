@@ -42,8 +42,13 @@ void Ops<KT>::apply_dot(const Lvl& L, int mode, const KT* x, KT* y, const RedBuf
   const int wonly = (mode == 0);
   if (mac3_level(L) && !GKB_VARMU(L) && x) k_mac3<KT, 1, true><<<mac3_grid(L), dim3(BX, BY), 0, s>>>(L, wonly, x, nullptr, y, red, fin, st, nullptr);
   else if (mac2_level<KT>(L) && x) {
-    if (GKB_VARMU(L)) k_mac2<KT, true><<<mac2_grid<KT>(L), dim3(BX, BY), 0, s>>>(L, wonly, x, y, red, fin, st);
-    else k_mac2<KT, false><<<mac2_grid<KT>(L), dim3(BX, BY), 0, s>>>(L, wonly, x, y, red, fin, st);
+    if constexpr (sizeof(KT) == 4) {
+      if (GKB_VARMU(L)) {
+        k_mac2<KT, true><<<mac2_grid<KT>(L), dim3(BX, BY), 0, s>>>(L, wonly, x, y, red, fin, st);
+        return;
+      }
+    }
+    k_mac2<KT, false><<<mac2_grid<KT>(L), dim3(BX, BY), 0, s>>>(L, wonly, x, y, red, fin, st);
   } else if (GKB_VARMU(L)) k_mac_tile<KT, true, 1, true><<<face_grid(L), dim3(BX, BY), 0, s>>>(L, wonly, x, nullptr, y, red, fin, st, nullptr);
   else k_mac_tile<KT, false, 1, true><<<face_grid(L), dim3(BX, BY), 0, s>>>(L, wonly, x, nullptr, y, red, fin, st, nullptr);
 }

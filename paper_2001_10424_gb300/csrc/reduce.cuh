@@ -23,28 +23,21 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// sums over the block of v[0..NV-1], value i to lane 0 of warp i. Through
-// shared memory: a warp adds the block's values eight (or so) to a lane, then
-// across its lanes; shuffles in every warp first would issue four times as
-// many FP64 additions, each of which holds the SM's FP64 unit for 16 cycles
-// (1024^2 product with dot, 4257 blocks: tile kernel 42.4 -> 41.3 us; in FP64 78.9 -> 72.1 us).
+// sums over the block (of at most 256 threads) of v[0..NV-1], value i to lane 0
+// of warp i. Through shared memory: a warp adds the block's values eight (or
+// so) to a lane, then across its lanes; shuffles in every warp first would
+// issue four times as many FP64 additions, each of which holds the SM's FP64
+// unit for 16 cycles (1024^2 product with dot, 4257 blocks: tile kernel 42.4 ->
+// 41.3 us; in FP64 78.9 -> 72.1 us).
 template <int NV>
 __device__ __forceinline__ double block_sum(const double (&v)[NV], double (*sh)[256], int tid, int nthr) {
   const int lane = tid & 31, warp = tid >> 5;
 #pragma unroll
-  for (int i = 0; i < NV; ++i)
-    if (tid < 256) sh[i][tid] = v[i];
-  for (int base = 256; base < nthr; base += 256) {  // blocks of more than 256 threads
-    __syncthreads();
-    if (tid >= base && tid < base + 256)
-#pragma unroll
-      for (int i = 0; i < NV; ++i) sh[i][tid - base] += v[i];
-  }
+  for (int i = 0; i < NV; ++i) sh[i][tid] = v[i];
   __syncthreads();
   double s = 0.0;
   if (warp < NV) {
-    const int n = nthr < 256 ? nthr : 256;
-    for (int t = lane; t < n; t += 32) s += sh[warp][t];
+    for (int t = lane; t < nthr; t += 32) s += sh[warp][t];
     s = warp_sum(s);
   }
   return s;

@@ -1535,7 +1535,6 @@ void Solver::set_problem(const gkb_grid* g, const double* viscosity, double mu0_
   }
   L64.mu0 = viscosity ? 1.0 : mu0;
   L64.sym = symgrad ? 1 : 0;
-  L64.fast = fast64() ? 1 : 0;
   finish_level(L64);
   Compact cmp = make_compact(L64);
   m = cmp.m;
