@@ -24,6 +24,7 @@ int guarded(gkb_handle h, F&& fn) {
     explicit ProfBind(gkb::Profiler* p) { gkb::g_prof = p; }
     ~ProfBind() { gkb::g_prof = nullptr; }
   } bind(&h->s.prof);
+  const gkb::CallBind call(h->s.stream);
   try {
     cudaError_t e = cudaSetDevice(h->device);
     if (e != cudaSuccess) {

@@ -435,6 +435,7 @@ struct Lockstep::Impl {
     store.emplace_back();
     store.back().alloc(v.size() * sizeof(J));
     GKB_CUDA(cudaMemcpy(store.back().p, v.data(), v.size() * sizeof(J), cudaMemcpyHostToDevice));
+    order_after_legacy();
     return (const J*)store.back().p;
   }
   const unsigned* put_map(const std::vector<unsigned>& m) {
@@ -443,6 +444,7 @@ struct Lockstep::Impl {
     store.emplace_back();
     store.back().alloc(m.size() * sizeof(unsigned));
     GKB_CUDA(cudaMemcpy(store.back().p, m.data(), m.size() * sizeof(unsigned), cudaMemcpyHostToDevice));
+    order_after_legacy();
     const unsigned* d = (const unsigned*)store.back().p;
     maps.emplace(m, d);
     return d;
@@ -1211,6 +1213,7 @@ Lockstep::Lockstep(Solver* const* S, int count, cudaStream_t cap1, cudaStream_t 
   M.cp.alloc(count);
   GKB_CUDA(cudaMemcpy(M.sp.p, sp.data(), count * sizeof(GkbState*), cudaMemcpyHostToDevice));
   GKB_CUDA(cudaMemcpy(M.cp.p, cp.data(), count * sizeof(CgState*), cudaMemcpyHostToDevice));
+  order_after_legacy();
   int* a = M.state.p;
   Flat& f = M.F;
   f.S = M.sp.p;

@@ -25,6 +25,21 @@
 namespace gkb {
 
 thread_local Profiler* g_prof = nullptr;
+thread_local CallStream g_call;
+
+void order_after_legacy() {
+  if (!g_call.known) {
+    GKB_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+    return;
+  }
+  if (g_call.s == nullptr || g_call.s == cudaStreamLegacy) return;
+  cudaEvent_t e;
+  GKB_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  cudaError_t rc = cudaEventRecord(e, cudaStreamLegacy);
+  if (rc == cudaSuccess) rc = cudaStreamWaitEvent(g_call.s, e, 0);
+  cudaEventDestroy(e);  // released once the wait is through
+  GKB_CUDA(rc);
+}
 
 void check_cuda(cudaError_t e, const char* what) {
   if (e != cudaSuccess) {

@@ -24,6 +24,24 @@ struct Error {
 void check_cuda(cudaError_t e, const char* what);
 #define GKB_CUDA(x) ::gkb::check_cuda((x), #x)
 
+// The stream that the call running on this thread launches on, set by the
+// entry points that have a handle or a network.
+struct CallStream {
+  bool known = false;
+  cudaStream_t s = nullptr;
+};
+extern thread_local CallStream g_call;
+struct CallBind {
+  CallStream before = g_call;
+  explicit CallBind(cudaStream_t s) { g_call = CallStream{true, s}; }
+  ~CallBind() { g_call = before; }
+};
+// What the host has put on the legacy stream so far (fills, copies) comes
+// before what the call launches from here on: the call's stream waits for it,
+// or the host does where that stream is not known. Nothing to do on the legacy
+// stream itself.
+void order_after_legacy();
+
 template <typename T>
 struct DevBuf {
   T* p = nullptr;
@@ -47,12 +65,12 @@ struct DevBuf {
       throw Error{GKB_ERR_OOM, "cudaMalloc of " + std::to_string(count * sizeof(T)) + " bytes failed"};
     }
     n = count;
-    // the fill runs on the legacy stream, and returns before it is done: waited
-    // for, as the caller's kernels may run on a stream that does not wait for
-    // that one (the weight gradient's partial sums are allocated right before
-    // the kernel that writes them)
+    // the fill runs on the legacy stream, and returns before it is done: ordered
+    // before the caller's kernels, which may run on a stream that does not wait
+    // for that one (the weight gradient's partial sums are allocated right
+    // before the kernel that writes them)
     GKB_CUDA(cudaMemset(p, 0, count * sizeof(T)));
-    GKB_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+    order_after_legacy();
   }
   void release() {
     if (p) cudaFree(p);

@@ -1301,6 +1301,7 @@ namespace {
 template <class F>
 int unet_guard(gkb_unet h, F&& fn) {
   if (!h) return GKB_ERR_INVALID_ARG;
+  const gkb::CallBind call(h->u.stream);
   try {
     if (cudaSetDevice(h->device) != cudaSuccess) {
       (void)cudaGetLastError();
@@ -1342,6 +1343,7 @@ int gkb_unet_create(gkb_unet* out, int c_in, int c1, int c2, int c_out, unsigned
     delete h;
     return GKB_ERR_CUDA;
   }
+  h->u.stream = (cudaStream_t)stream;
   int rc = unet_guard(h, [&] {
     h->u.init(c_in, c1, c2, c_out, seed, (cudaStream_t)stream);
     gkb::check_cuda(cudaStreamSynchronize((cudaStream_t)stream), "init");
