@@ -105,27 +105,26 @@ __device__ __forceinline__ void to_f64(const float (&v)[N], double (&o)[N]) {
   }
 }
 
-// 1 / b as its rounded value and the rest of it (the remainder 1 - b y of a
-// correctly rounded y is exact)
-struct Recip {
-  double y, lo;
-};
-__device__ __forceinline__ Recip recip(double b) {
-  const double y = 1.0 / b;
-  return {y, y * fma(-b, y, 1.0)};
-}
-// a / b, rounded as the division rounds, from r = recip(b) (Markstein: with
-// y = 1 / b rounded to nearest and a q less than an ulp off a / b, the remainder
-// a - b q is exact and q plus its quotient by y rounds correctly). a y alone
-// can be 1.5 ulps off; with the rest of 1 / b q is within 0.5 and a little.
+// a / b, rounded as the division rounds, from y = 1 / b rounded to nearest.
+// Let a, b and the quotient Q have p-bit integers as significands (p = 53) and
+// y be off 1 / b by t units of its own last place, |t| <= 1/2. Then q = a y is
+// off Q by at most |a t| 2^(1-p) and half a unit.
+// * Significand of a not below b's: q is less than a unit off, the remainder
+//   a - b q is exact and one correction rounds correctly (Markstein).
+// * Below: q is less than 1.5 units off, and the remainder may need p + 1 bits.
+//   Its rounding and y's error then move Q by at most 1.5 x 2^(1-p), which can
+//   only cross a midpoint that lies k / (2 b) from Q with k <= 5; q is 1.5 units
+//   from such a Q less k / (2 b). That takes |a t| 2^(1-p) > 1 - k / (2 b), so
+//   t near 1/2 and 2 (2^p - a) + (2^p - b)^2 <= 5, that is a = 2^p - 2,
+//   b = 2^p - 1, whose quotient lies next to an integer.
 // Outside the exponents where no term under- or overflows: the division itself.
-__device__ __forceinline__ double div_by(double a, double b, Recip r) {
+__device__ __forceinline__ double div_by(double a, double b, double y) {
   // biased exponents within 500 of 1 (integer tests: a comparison on the FP64
   // unit costs as much as a multiply-add)
   const unsigned ea = ((unsigned)__double2hiint(a) >> 20) & 0x7ff, eb = ((unsigned)__double2hiint(b) >> 20) & 0x7ff;
   if (ea - 523u > 1000u || eb - 523u > 1000u) return a / b;
-  const double q = fma(a, r.y, a * r.lo);
-  return fma(fma(-b, q, a), r.y, q);
+  const double q = a * y;
+  return fma(fma(-b, q, a), y, q);
 }
 
 __device__ __forceinline__ Blk native_blk() {

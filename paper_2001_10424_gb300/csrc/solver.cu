@@ -1005,9 +1005,9 @@ __global__ void __launch_bounds__(SB) k_cg_cluster(Lvl L, const double* __restri
 // the chain of link sums); rows packed into as few warps as hold them; both
 // sums reduced together; a ninth warp for the scalars, which works out
 // 1 / gamma and 1 / alpha while the others update and multiply, so that two
-// of the recurrence's three divisions become four operations each. The
+// of the recurrence's three divisions become three operations each. The
 // shares, the operations and the order of every sum are those of
-// k_cg_cluster, so the bits are too. 32 x 32 channel: 9.3 -> 5.2 us per
+// k_cg_cluster, so the bits are too. 32 x 32 channel: 9.3 -> 5.1 us per
 // iteration.
 constexpr int CGS_E = 4;            // entries of its share per thread
 constexpr int CGS_F = 3;            // rows per thread
@@ -1305,8 +1305,7 @@ __global__ void __launch_bounds__(CGS_NT) k_cg_cluster_sm(const __grid_constant_
   cl.sync();  // r complete
   // the recurrence's scalars live in the scalars' warp of every block (the
   // same values), with the reciprocals of gamma and alpha
-  double gamma = 0.0, delta = 0.0, gamma_prev = 0.0, alpha = 0.0, stop_at = 0.0;
-  Recip y_gamma{0.0, 0.0}, y_alpha{0.0, 0.0};
+  double gamma = 0.0, delta = 0.0, gamma_prev = 0.0, alpha = 0.0, y_gamma = 0.0, y_alpha = 0.0, stop_at = 0.0;
   int it = 0, status = ST_OK;
   auto step = [&]() {  // the next alpha and beta, or the end
     int stop = 0;
@@ -1361,8 +1360,8 @@ __global__ void __launch_bounds__(CGS_NT) k_cg_cluster_sm(const __grid_constant_
     } else {
       cl.barrier_arrive();
       if (ctl && lane == 0) {  // for the next iteration's quotients
-        y_gamma = recip(gamma);
-        y_alpha = recip(alpha);
+        y_gamma = 1.0 / gamma;
+        y_alpha = 1.0 / alpha;
       }
       __syncwarp();
     }
@@ -1986,10 +1985,10 @@ void Solver::launch_cg_block(const double* fpad, double* xpad, cudaStream_t s) {
   const bool var = L64.mu64 != nullptr;
   // every vector on chip where a block's copy of r and the threads' entries
   // have room (us per iteration, k_cg_cluster -> on chip: 2D constant viscosity
-  // 32^2 9.3 -> 5.3, 62 x 60 11.2 -> 7.0; variable 16^2 10.2 -> 5.0, 62 x 60
-  // 12.0 -> 7.3; 3D constant 4^3 12.3 -> 6.2, 10^3 13.6 -> 7.1, 31 x 7 x 5
-  // 11.4 -> 8.2; variable 4^3 14.7 -> 6.2, 10^3 16.1 -> 7.3, 31 x 7 x 5 13.5 ->
-  // 8.5); kernel_variant 1 keeps the general kernel, which has the same bits
+  // 32^2 9.3 -> 5.2, 62 x 60 11.2 -> 6.8; variable 16^2 10.2 -> 4.7, 62 x 60
+  // 12.0 -> 7.2; 3D constant 4^3 12.3 -> 6.2, 10^3 13.6 -> 7.0, 31 x 7 x 5
+  // 11.4 -> 8.1; variable 4^3 14.7 -> 6.2, 10^3 16.1 -> 7.2, 31 x 7 x 5 13.5 ->
+  // 8.4); kernel_variant 1 keeps the general kernel, which has the same bits
   constexpr size_t max_sm = 190 * 1024;
   const bool d3 = L64.dim == 3;
   auto sm_fn = d3 ? (var ? k_cg_cluster_sm<3, true> : k_cg_cluster_sm<3, false>)

@@ -43,7 +43,7 @@ __global__ void k_div(int kind, long long n, unsigned long long* bad) {
     a = fma(b, q, b * half);
     a = bits((uint64_t)__double_as_longlong(a) + (v >> 60 & 3) - 1);  // and its neighbours
   }
-  if (!same(gkb::div_by(a, b, gkb::recip(b)), a / b)) atomicAdd(bad, 1ull);
+  if (!same(gkb::div_by(a, b, 1.0 / b), a / b)) atomicAdd(bad, 1ull);
 }
 
 // groups of four floats: every bit pattern in turn beside three hashed ones
