@@ -494,7 +494,7 @@ def roofline(gk, torch, wk, args, form, hbm_peak, peak_kind):
     B.destroy()
     how = "%d problem(s), profiled host-sequenced solve" % n_profiled
     run_ms = None
-    if wk.dim == 2:
+    if wk.dim == 2 and wk.inner != gk.GKB_INNER_CG:
         # the classes above are those of a V-cycle's separate steps, which have
         # algorithmic bytes and flops of their own; a 2D solve fuses a level's
         # steps into legs: the time per class of the launches that it makes
