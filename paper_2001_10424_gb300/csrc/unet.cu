@@ -636,8 +636,8 @@ __global__ void __launch_bounds__(256, 2) k_wgrad(const WgradArgs A) {
   if (tid < co * A.bgroups) A.bpart[(long long)blockIdx.x * co * A.bgroups + tid] = bsum;
 }
 
-// The rows of partials added in a fixed order: WG_RG row groups of a block
-// (rows k, k + WG_RG, ...), then the groups in FP64. Blocks [0, wblocks): the
+// The rows of partials added in a fixed order: RG row groups of a block (rows k,
+// k + RG, ...), then the groups in FP64. Blocks [0, wblocks): the
 // weights' sums, from the order of a row (T threads of cow outputs) to
 // [tap][ci][co]; the others: the biases'.
 //
@@ -647,28 +647,32 @@ __global__ void __launch_bounds__(256, 2) k_wgrad(const WgradArgs A) {
 // a thousand rows held that unit for 40 to 100 us a layer (1 x 512^2: 1.12 ms
 // for the nine layers' weight gradients, now 0.81). Sums that leave FP32's
 // range are formed in FP64.
-constexpr int WG_RC = 8, WG_RG = 32;  // columns and row groups of a block
+// A block takes RC columns: 8 in 32 row groups, or 32 in 8, which leaves a
+// quarter of the FP64 additions, where there are at most 256 rows (128 rows of
+// 9216 sums: 9.1 -> 5.6 us).
 struct ReduceArgs {
   const float* partial;
   const double* bpart;
   float* out;
   int nrows, brows, cin, co, cow, wblocks;
 };
-__global__ void __launch_bounds__(WG_RC* WG_RG) k_reduce_wgrad(const ReduceArgs A) {
-  __shared__ double sh[WG_RC * WG_RG / 32][WG_RC];
-  const int c = threadIdx.x % WG_RC, k = threadIdx.x / WG_RC;
+template <int RC>
+__global__ void __launch_bounds__(256) k_reduce_wgrad(const ReduceArgs A) {
+  constexpr int RG = 256 / RC;
+  __shared__ double sh[8][RC];
+  const int c = threadIdx.x % RC, k = threadIdx.x / RC;
   const bool bias = (int)blockIdx.x >= A.wblocks;
-  const int t = ((int)blockIdx.x - (bias ? A.wblocks : 0)) * WG_RC + c;
+  const int t = ((int)blockIdx.x - (bias ? A.wblocks : 0)) * RC + c;
   const int nw = 9 * A.cin * A.co, nt = bias ? A.co : nw;
   double s = 0.0;
   if (t < nt) {
     if (bias) {
 #pragma unroll 8
-      for (int b = k; b < A.brows; b += WG_RG) s += A.bpart[(long long)b * A.co + t];
+      for (int b = k; b < A.brows; b += RG) s += A.bpart[(long long)b * A.co + t];
     } else {
       float hi = 0.f, lo = 0.f;
 #pragma unroll 16
-      for (int b = k; b < A.nrows; b += WG_RG) {
+      for (int b = k; b < A.nrows; b += RG) {
         const float v = A.partial[(long long)b * nw + t];
         const float z = hi + v, w = z - hi;
         lo += (hi - (z - w)) + (v - w);
@@ -677,15 +681,16 @@ __global__ void __launch_bounds__(WG_RC* WG_RG) k_reduce_wgrad(const ReduceArgs 
       s = (double)hi + (double)lo;
       if (!isfinite(s)) {
         s = 0.0;
-        for (int b = k; b < A.nrows; b += WG_RG) s += A.partial[(long long)b * nw + t];
+        for (int b = k; b < A.nrows; b += RG) s += A.partial[(long long)b * nw + t];
       }
     }
   }
-  for (int o = 16; o >= WG_RC; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) < WG_RC) sh[threadIdx.x >> 5][c] = s;
+#pragma unroll
+  for (int o = 16; o >= RC; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) < RC) sh[threadIdx.x >> 5][c] = s;
   __syncthreads();
   if (k == 0 && t < nt) {
-    for (int q = 1; q < WG_RC * WG_RG / 32; ++q) s += sh[q][c];
+    for (int q = 1; q < 8; ++q) s += sh[q][c];
     int at = nw + t;
     if (!bias) {
       const int T = A.cin * (A.co / A.cow), o = t % A.cow, r = t / A.cow % T, tap = t / (A.cow * T);
@@ -1005,7 +1010,7 @@ const float* Unet::forward(UnetAct& A, const float* x, int n, int h, int w, bool
 // groups count), so that about 1024 rows of a group are written and added up.
 // Against one sum per thread over all its pixels (128 to 2048), which was up
 // to five times as far off as the 8-pixel sums, a training step of 1 x 128^2
-// takes 0.82 ms in place of 0.76, one of 8 x 512^2 9.74 in place of 9.95.
+// takes 0.81 ms in place of 0.76, one of 8 x 512^2 9.70 in place of 9.95.
 constexpr int WG_ROWS = 1024;
 // Outputs per thread: 4 (registers for 24 warps per SM), 8 where 4 would need
 // more threads than a block has, 2 where so few channels leave threads idle.
@@ -1062,9 +1067,12 @@ static void conv_bwd_w(Unet& U, int li, In2 in, const float* dpre, int n, int h,
   else if (cow == 3) k_wgrad<3><<<nblk, nt, sm, s>>>(A);
   else if (cow == 2) k_wgrad<2><<<nblk, nt, sm, s>>>(A);
   else k_wgrad<1><<<nblk, nt, sm, s>>>(A);
-  const int wb = (int)((L.nw() + WG_RC - 1) / WG_RC);
-  const ReduceArgs R{U.wpart.p, U.bpart.p, U.grads.p + L.off, nblk * A.groups * A.rows, nblk * A.bgroups, L.cin, L.cout, cow, wb};
-  k_reduce_wgrad<<<wb + (L.cout + WG_RC - 1) / WG_RC, WG_RC * WG_RG, 0, s>>>(R);
+  ReduceArgs R{U.wpart.p, U.bpart.p, U.grads.p + L.off, nblk * A.groups * A.rows, nblk * A.bgroups, L.cin, L.cout, cow, 0};
+  const int rc = R.nrows <= 256 ? 32 : 8;
+  R.wblocks = (int)((L.nw() + rc - 1) / rc);
+  const int blocks = R.wblocks + (L.cout + rc - 1) / rc;
+  if (rc == 32) k_reduce_wgrad<32><<<blocks, 256, 0, s>>>(R);
+  else k_reduce_wgrad<8><<<blocks, 256, 0, s>>>(R);
   GKB_CUDA(cudaGetLastError());
 }
 
