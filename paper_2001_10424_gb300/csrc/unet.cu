@@ -467,12 +467,13 @@ __global__ void __launch_bounds__(TCT) k_conv_fwd_tc(In2 in, const __nv_bfloat16
 // the gradients of a warp are consecutive words or broadcasts). The thread
 // groups of a block share its rows of pixels.
 //
-// An FP32 sum ends after `chain` pixels (wgrad_shape): the thread adds it to
-// its row of partials and starts again. A row holds 9 x T x COW values at
+// An FP32 sum ends after `chain` pixels (wgrad_shape); `per_row` of them are
+// added up beside the running one (TWO: more than one) and leave as the
+// thread's part of a row of partials. A row holds 9 x T x COW values at
 // (tap T + thread) COW + output, so that a warp's sums are consecutive there.
-// On 8 images of 512^2: 48 -> 16 1.48 ms (20 TFLOP/s; staging the bilinear
-// input costs as much as the sums), 16 -> 16 0.48 ms, 64 -> 32 at half
-// resolution 0.72 ms; the nine layers with their reductions 4.0 ms, a thread
+// On 8 images of 512^2: 48 -> 16 1.51 ms (19 TFLOP/s; staging the bilinear
+// input costs as much as the sums), 16 -> 16 0.50 ms, 64 -> 32 at half
+// resolution 0.68 ms; the nine layers with their reductions 4.0 ms, a thread
 // per weight on 8-pixel patches took 44 ms.
 constexpr int WGC = 32;  // columns of a tile
 struct WgradArgs {
@@ -486,8 +487,8 @@ struct WgradArgs {
   int bgroups;               // rows of bpart of a block
 };
 
-template <int COW>
-__global__ void __launch_bounds__(256, 2) k_wgrad(const WgradArgs A) {
+template <int COW, int NTM, bool TWO>
+__global__ void __launch_bounds__(NTM, 512 / NTM) k_wgrad(const WgradArgs A) {
   extern __shared__ __align__(16) float wg_sm[];
   const int cin = A.cin, co = A.co, T = cin * (co / COW), NT = blockDim.x, tid = threadIdx.x;
   const int xrow = (WGC + 2) * cin;
@@ -504,31 +505,48 @@ __global__ void __launch_bounds__(256, 2) k_wgrad(const WgradArgs A) {
   const int nw = 9 * cin * co;
   float* const rows = A.partial + ((long long)(blockIdx.x * A.groups + g) * A.rows) * nw + (long long)r * COW;
   int done = 0, sums = 0;  // pixels of the current sum, sums written
+  float tot[TWO ? 9 : 1][TWO ? COW : 1];  // the row's sums so far
+  if constexpr (TWO) {
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
+#pragma unroll
+      for (int o = 0; o < COW; ++o) tot[q][o] = 0.f;
+  }
   auto flush = [&]() {
-    float* out = rows + (long long)(sums / A.per_row) * nw;
-    const bool first = sums % A.per_row == 0;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      float* d = out + q * T * COW;
-      if constexpr (COW % 4 == 0) {
-#pragma unroll
-        for (int o = 0; o < COW; o += 4) {
-          float4 v = make_float4(acc[q][o], acc[q][o + 1], acc[q][o + 2], acc[q][o + 3]);
-          if (!first) {
-            const float4 u = *reinterpret_cast<const float4*>(d + o);
-            v = make_float4(u.x + v.x, u.y + v.y, u.z + v.z, u.w + v.w);
-          }
-          *reinterpret_cast<float4*>(d + o) = v;
-        }
-      } else {
-#pragma unroll
-        for (int o = 0; o < COW; ++o) d[o] = first ? acc[q][o] : d[o] + acc[q][o];
-      }
-#pragma unroll
-      for (int o = 0; o < COW; ++o) acc[q][o] = 0.f;
-    }
     done = 0;
     ++sums;
+    if constexpr (TWO) {
+#pragma unroll
+      for (int q = 0; q < 9; ++q)
+#pragma unroll
+        for (int o = 0; o < COW; ++o) {
+          acc[q][o] += tot[q][o];
+          tot[q][o] = acc[q][o];
+        }
+    }
+    if (!TWO || sums % A.per_row == 0) {
+      float* out = rows + (long long)((sums - 1) / A.per_row) * nw;
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        float* d = out + q * T * COW;
+        if constexpr (COW % 4 == 0) {
+#pragma unroll
+          for (int o = 0; o < COW; o += 4)
+            *reinterpret_cast<float4*>(d + o) = make_float4(acc[q][o], acc[q][o + 1], acc[q][o + 2], acc[q][o + 3]);
+        } else {
+#pragma unroll
+          for (int o = 0; o < COW; ++o) d[o] = acc[q][o];
+        }
+        if constexpr (TWO) {
+#pragma unroll
+          for (int o = 0; o < COW; ++o) tot[q][o] = 0.f;
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
+#pragma unroll
+      for (int o = 0; o < COW; ++o) acc[q][o] = 0.f;
   };
   const int tx = (A.wd + WGC - 1) / WGC, tyn = (A.h + A.ty - 1) / A.ty;
   const int t1 = min(A.tiles, (int)(blockIdx.x + 1) * A.per_block);
@@ -647,19 +665,21 @@ __global__ void __launch_bounds__(256, 2) k_wgrad(const WgradArgs A) {
 // a thousand rows held that unit for 40 to 100 us a layer (1 x 512^2: 1.12 ms
 // for the nine layers' weight gradients, now 0.81). Sums that leave FP32's
 // range are formed in FP64.
-// A block takes RC columns: 8 in 32 row groups, or 32 in 8, which leaves a
-// quarter of the FP64 additions, where there are at most 256 rows (128 rows of
-// 9216 sums: 9.1 -> 5.6 us).
+// A block of NT threads takes RC columns: 8 in 32 row groups; 32 in 8, which
+// leaves a quarter of the FP64 additions, where there are at most 256 rows (128
+// rows of 9216 sums: 9.1 -> 5.6 us); or 8 in 128, a quarter of the loads one
+// after another, where the columns give few blocks (4096 rows of 432 sums:
+// 21 -> 14 us).
 struct ReduceArgs {
   const float* partial;
   const double* bpart;
   float* out;
   int nrows, brows, cin, co, cow, wblocks;
 };
-template <int RC>
-__global__ void __launch_bounds__(256) k_reduce_wgrad(const ReduceArgs A) {
-  constexpr int RG = 256 / RC;
-  __shared__ double sh[8][RC];
+template <int RC, int NT>
+__global__ void __launch_bounds__(NT) k_reduce_wgrad(const ReduceArgs A) {
+  constexpr int RG = NT / RC;
+  __shared__ double sh[NT / 32][RC];
   const int c = threadIdx.x % RC, k = threadIdx.x / RC;
   const bool bias = (int)blockIdx.x >= A.wblocks;
   const int t = ((int)blockIdx.x - (bias ? A.wblocks : 0)) * RC + c;
@@ -690,7 +710,7 @@ __global__ void __launch_bounds__(256) k_reduce_wgrad(const ReduceArgs A) {
   if ((threadIdx.x & 31) < RC) sh[threadIdx.x >> 5][c] = s;
   __syncthreads();
   if (k == 0 && t < nt) {
-    for (int q = 1; q < 8; ++q) s += sh[q][c];
+    for (int q = 1; q < NT / 32; ++q) s += sh[q][c];
     int at = nw + t;
     if (!bias) {
       const int T = A.cin * (A.co / A.cow), o = t % A.cow, r = t / A.cow % T, tap = t / (A.cow * T);
@@ -900,8 +920,8 @@ void Unet::init(int cin, int k1, int k2, int cout, unsigned long long seed, cuda
   allow_fwd<8, 2, 1>(48);
   allow_fwd<8, 4, 2>(64);
   allow_fwd<8, 4, 1>(64);
-  GKB_CUDA(cudaFuncSetAttribute(k_wgrad<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
-  GKB_CUDA(cudaFuncSetAttribute(k_wgrad<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
+  for (auto f : {k_wgrad<4, 256, false>, k_wgrad<4, 256, true>, k_wgrad<4, 512, false>, k_wgrad<4, 512, true>})
+    GKB_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
   bf16_stale = true;
   adam_t = 0;
 }
@@ -1004,19 +1024,20 @@ const float* Unet::forward(UnetAct& A, const float* x, int n, int h, int w, bool
 // Rounding: an FP32 sum of F terms leaves an error of about sqrt(F / 2) units
 // of its last place, and the sums of R / F of them in a row sqrt(R / (2 F)).
 // The bound kept is that of sums over 8 pixels added up by 304 blocks,
-// 8 + N / 2432 for F: F is the largest power of two below 3/4 of it, which
-// leaves room for the additions into a row, at least 8. A row takes
-// R = N / 1024 pixels per thread group (a power of two, at least F; up to four
-// groups count), so that about 1024 rows of a group are written and added up.
-// Against one sum per thread over all its pixels (128 to 2048), which was up
-// to five times as far off as the 8-pixel sums, a training step of 1 x 128^2
-// takes 0.81 ms in place of 0.76, one of 8 x 512^2 9.70 in place of 9.95.
-constexpr int WG_ROWS = 1024;
-// Outputs per thread: 4 (registers for 24 warps per SM), 8 where 4 would need
-// more threads than a block has, 2 where so few channels leave threads idle.
+// 8 + N / 2432 for F: F is the largest power of two below 0.65 of it, which
+// leaves room for the additions into a row and for neighbouring terms that are
+// not independent, at least 8. A row takes R = N / 1280 pixels of a thread group
+// (a power of two, at least F; up to four groups count), so that 640 to 1280
+// rows of a group are written and added up.
+// One sum per thread over all its pixels (128 to 2048) was up to five times as
+// far off. Training steps against it: 1 x 64^2 0.74 -> 0.70 ms, 1 x 128^2 0.77
+// -> 0.75, 1 x 256^2 0.94 -> 0.99, 8 x 96^2 1.07 -> 1.14, 1 x 512^2 1.89 -> 1.79,
+// 8 x 512^2 9.97 -> 9.72.
+constexpr int WG_ROWS = 1280;
+// Outputs per thread: 4 (two sums of each: 16 warps of 128 registers per SM; 64
+// -> 32 takes blocks of 512 threads), 2 where so few channels leave threads idle.
 static int wgrad_cow(const ConvLayer& L) {
   if (L.cout % 8) return L.cout;
-  if (L.cin * L.cout / 4 > 256) return 8;
   return L.cin * L.cout / 4 < 32 ? 2 : 4;
 }
 static WgradArgs wgrad_shape(const ConvLayer& L, int n, int h, int w) {
@@ -1028,15 +1049,19 @@ static WgradArgs wgrad_shape(const ConvLayer& L, int n, int h, int w) {
   A.wd = w;
   const int T = L.cin * (L.cout / wgrad_cow(L));
   A.groups = std::max(1, std::min(8, 256 / T));
+  // rows of a tile: four (a halo of two more), or one of each group where that
+  // leaves SMs without a block
   A.ty = std::max(4, A.groups);
-  A.tiles = n * ((w + WGC - 1) / WGC) * ((h + A.ty - 1) / A.ty);
+  auto tiles = [&] { return n * ((w + WGC - 1) / WGC) * ((h + A.ty - 1) / A.ty); };
+  if (tiles() < 152) A.ty = A.groups;
+  A.tiles = tiles();
   const long long N = (long long)n * h * w;
   A.chain = 8;
-  while (2 * A.chain <= 6 + 3 * N / 9728) A.chain *= 2;
+  while (2 * A.chain <= 0.65 * (8 + N / 2432.0)) A.chain *= 2;
+  const int px = WGC * A.ty / A.groups;  // pixels of a tile per thread
   long long row = A.chain;  // pixels of a row of partials
   while (row * WG_ROWS * std::min(A.groups, 4) < N) row *= 2;
   A.per_row = (int)(row / A.chain);
-  const int px = WGC * A.ty / A.groups;  // pixels of a tile per thread
   A.per_block = (int)std::max(1LL, row / px);
   A.rows = (int)std::max(1LL, px / row);
   const int runs = (WGC * A.ty + A.chain - 1) / A.chain;  // runs of dpre sums in a tile
@@ -1062,17 +1087,23 @@ static void conv_bwd_w(Unet& U, int li, In2 in, const float* dpre, int n, int h,
   const size_t sm = tile * sizeof(float);
   cudaStream_t s = U.stream;
   ProfScope ps_(GKB_KC_UNET, s, (long long)n * h * w);
-  if (cow == 8) k_wgrad<8><<<nblk, nt, sm, s>>>(A);
-  else if (cow == 4) k_wgrad<4><<<nblk, nt, sm, s>>>(A);
-  else if (cow == 3) k_wgrad<3><<<nblk, nt, sm, s>>>(A);
-  else if (cow == 2) k_wgrad<2><<<nblk, nt, sm, s>>>(A);
-  else k_wgrad<1><<<nblk, nt, sm, s>>>(A);
+  const bool two = A.per_row > 1;
+#define GKB_WG(COW, NTM)                                  \
+  if (two) k_wgrad<COW, NTM, true><<<nblk, nt, sm, s>>>(A); \
+  else k_wgrad<COW, NTM, false><<<nblk, nt, sm, s>>>(A)
+  if (cow == 4 && nt > 256) { GKB_WG(4, 512); }
+  else if (cow == 4) { GKB_WG(4, 256); }
+  else if (cow == 3) { GKB_WG(3, 256); }
+  else if (cow == 2) { GKB_WG(2, 256); }
+  else { GKB_WG(1, 256); }
+#undef GKB_WG
   ReduceArgs R{U.wpart.p, U.bpart.p, U.grads.p + L.off, nblk * A.groups * A.rows, nblk * A.bgroups, L.cin, L.cout, cow, 0};
   const int rc = R.nrows <= 256 ? 32 : 8;
   R.wblocks = (int)((L.nw() + rc - 1) / rc);
   const int blocks = R.wblocks + (L.cout + rc - 1) / rc;
-  if (rc == 32) k_reduce_wgrad<32><<<blocks, 256, 0, s>>>(R);
-  else k_reduce_wgrad<8><<<blocks, 256, 0, s>>>(R);
+  if (rc == 32) k_reduce_wgrad<32, 256><<<blocks, 256, 0, s>>>(R);
+  else if (blocks < 304) k_reduce_wgrad<8, 1024><<<blocks, 1024, 0, s>>>(R);
+  else k_reduce_wgrad<8, 256><<<blocks, 256, 0, s>>>(R);
   GKB_CUDA(cudaGetLastError());
 }
 
